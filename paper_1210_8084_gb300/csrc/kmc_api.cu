@@ -56,6 +56,7 @@ struct kmc_handle {
     uint32_t n_stage_tiles = 0;
     int stage_cap = 0, stage_rows = 0, stage_stride = 0, stage_pair_cap = 0, any_direct = 1, any_tiled = 0;
     int any_plain_tiled = 0;
+    int filtered = 0, filter_chi = 0, filter_split = 0;   // filtered search (see Bufs)
     int cbin_moments = 0;   // moments one warp per c-bin (every c-bin: at most kCbinRows runs of search cells)
     int tile_threads = 256, tile_cap = 1536, tile_split = 1, tile_prune = 1;
     int64_t n_bins = 0, bins_per_inst = 0;
@@ -141,6 +142,9 @@ Bufs<T> make_bufs(const kmc_handle* h) {
     b.any_direct = h->any_direct;
     b.any_tiled = h->any_tiled;
     b.any_plain_tiled = h->any_plain_tiled;
+    b.filtered = h->filtered;
+    b.filter_chi = h->filter_chi;
+    b.filter_split = h->filter_split;
     b.dsmc = (h->cfg.flags & KMC_FLAG_DSMC) ? 1 : 0;
     b.radial = (h->cfg.flags & KMC_FLAG_RADIAL_MOMENT) ? 1 : 0;
     b.tile_threads = h->tile_threads;
@@ -166,8 +170,9 @@ cudaError_t enqueue_step(kmc_handle* h, int want_moments, cudaEvent_t* ev = null
     if ((e = mark(KMC_PHASE_SEARCH)) != cudaSuccess) return e;
     if (b.dsmc) {   // random partners inside each c-bin instead of the closest-approach search
         if ((e = launch_dsmc<T>(b, s)) != cudaSuccess) return e;
-    } else if ((e = launch_search<T>(b, s)) != cudaSuccess) {
-        return e;
+    } else {
+        if ((e = launch_search<T>(b, s)) != cudaSuccess) return e;
+        if (b.filtered && (e = launch_filtered_search<T>(b, s)) != cudaSuccess) return e;
     }
     if ((e = mark(KMC_PHASE_TILE)) != cudaSuccess) return e;
     if (!b.dsmc && (e = launch_tile_search<T>(b, s)) != cudaSuccess) return e;
@@ -335,6 +340,41 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
         I.M[d] = h->geo.n[d] * s[d];
         I.w[d] = h->geo.L[d] / (double)I.M[d];
     }
+}
+
+// Search of instance i where no option asks for a particular one: the filtered
+// search or one thread per particle, and the filtered search's form.  Estimates
+// per particle: `occ` is the particles' mean occupancy of their c-bin; `cand`
+// the candidates of the first step's window, `within` those inside the contact
+// distance (cut at the window), `passing` those that meet within an rms
+// displacement; `near` those one filter leaves (inside R and half a relative
+// displacement, about 1.1 vrms dt).
+// Binary32 looks at each pair once, its threshold then staying R^2, or, where many
+// candidates pass, at every home's whole window with a threshold that falls to
+// its closest candidate: twice the pairs, but few of them left (a twentieth on
+// the quadrant workload).  Binary64 always filters (its exact test runs at 1/64
+// of the binary32 rate), by criterion 1 too.
+void choose_filter(kmc_handle* h, InstDev& I, double vmax, double vrms, double occ) {
+    const double dt0 = (I.adaptive && vmax > 0.0) ? I.dx_min / vmax : I.dt;
+    const double R = sqrt(I.R2), reach = 1.001 * (R + 2.0 * vmax * dt0), rho = sqrt(I.R2 + 1.2 * vrms * vrms * dt0 * dt0);
+    double cand = occ, within = occ, near = occ;
+    for (int d = 0; d < h->dim; ++d) {
+        const double L = h->geo.L[d], bin = L / h->geo.n[d], widest = std::min(3.0 * bin, L);
+        const double win = (2.0 * ceil((reach + 1e-5 * L) / I.w[d]) + 1.0) * I.w[d];
+        cand *= std::min(win, widest) / bin;
+        within *= std::min(2.0 * R, widest) / bin;
+        near *= std::min(2.0 * rho, widest) / bin;
+    }
+    const double passing = within * (R > 0.0 ? std::min(1.0, vrms * dt0 / R) : 0.0);
+    I.sym = h->precision == 32 && passing <= kSymPassing ? 1 : 0;
+    // a ball in the cube of near; each pair once
+    double hits = I.sym ? 0.5 * near * (h->dim == 3 ? 0.52 : 0.79) : 0.05 * cand;
+    if (I.sym && hits > kChiHits && R > 1.5 * vrms * dt0 && vmax < 6.0 * vrms) {
+        h->filter_chi = 1;   // criterion 1 leaves about the passing ones
+        hits = std::min(hits, 4.0 * passing);
+    }
+    if (h->precision == 64) h->filter_chi = 1;
+    I.filtered = I.n > 0 && (h->precision == 64 || I.prune || filter_pays(cand, hits)) ? 1 : 0;
 }
 
 // Staged search plan (3-D only): a tile is tile_rows y-rows of one x-slab,
@@ -683,23 +723,24 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
     // search grid: per-instance vmax and densest c-bin of the initial state
     {
         uint32_t* hist = nullptr;
-        unsigned long long* vm = nullptr;
+        unsigned long long* vm = nullptr;   // bits of the largest |v|^2, then a sample's sums of |v|^2 and counts
         if ((rc = dev_alloc(h, (void**)&hist, sizeof(uint32_t) * (size_t)h->n_bins))) return bail(rc);
-        if ((rc = dev_alloc(h, (void**)&vm, sizeof(unsigned long long) * h->n_inst))) return bail(rc);
+        if ((rc = dev_alloc(h, (void**)&vm, 3 * sizeof(unsigned long long) * h->n_inst))) return bail(rc);
         std::vector<uint32_t> hist_h((size_t)h->n_bins, 0u);
-        std::vector<unsigned long long> vm_h(h->n_inst, 0ull);
+        std::vector<unsigned long long> vm_h(3 * (size_t)h->n_inst, 0ull);
         bool okc = cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)h->n_bins, h->stream) == cudaSuccess &&
-                   cudaMemsetAsync(vm, 0, sizeof(unsigned long long) * h->n_inst, h->stream) == cudaSuccess;
+                   cudaMemsetAsync(vm, 0, 3 * sizeof(unsigned long long) * h->n_inst, h->stream) == cudaSuccess;
         if (okc && n > 0) {
+            double* sample = (double*)(vm + h->n_inst);
             const cudaError_t e = h->precision == 64
-                                      ? launch_cbin_hist<double>(make_bufs<double>(h), hist, vm, h->stream)
-                                      : launch_cbin_hist<float>(make_bufs<float>(h), hist, vm, h->stream);
+                                      ? launch_cbin_hist<double>(make_bufs<double>(h), hist, vm, sample, h->stream)
+                                      : launch_cbin_hist<float>(make_bufs<float>(h), hist, vm, sample, h->stream);
             okc = e == cudaSuccess;
         }
         okc = okc &&
               cudaMemcpyAsync(hist_h.data(), hist, sizeof(uint32_t) * (size_t)h->n_bins, cudaMemcpyDeviceToHost,
                               h->stream) == cudaSuccess &&
-              cudaMemcpyAsync(vm_h.data(), vm, sizeof(unsigned long long) * h->n_inst, cudaMemcpyDeviceToHost,
+              cudaMemcpyAsync(vm_h.data(), vm, 3 * sizeof(unsigned long long) * h->n_inst, cudaMemcpyDeviceToHost,
                               h->stream) == cudaSuccess &&
               cudaStreamSynchronize(h->stream) == cudaSuccess;
         if (!okc) return bail(fail(h, KMC_ECUDA, "search-grid statistics failed"));
@@ -707,16 +748,26 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         std::vector<uint32_t> max_occ(h->n_inst, 0u);
         for (int i = 0; i < h->n_inst; ++i) {
             uint32_t mx = 0;
-            for (int64_t b = 0; b < h->bins_per_inst; ++b) mx = std::max(mx, hist_h[(size_t)(i * h->bins_per_inst + b)]);
+            uint64_t sq = 0;   // of the occupancies
+            const uint32_t* hist_i = hist_h.data() + (size_t)(i * h->bins_per_inst);
+            for (int64_t b = 0; b < h->bins_per_inst; ++b) {
+                mx = std::max(mx, hist_i[b]);
+                sq += (uint64_t)hist_i[b] * hist_i[b];
+            }
             max_occ[i] = mx;
             double v2;
             memcpy(&v2, &vm_h[i], sizeof(double));
             choose_subdivision(h, h->inst_h[i], sqrt(v2), mx);
+            double sample[2];
+            memcpy(sample, &vm_h[(size_t)h->n_inst + 2 * i], sizeof(sample));
+            choose_filter(h, h->inst_h[i], sqrt(v2), sample[1] > 0.0 ? sqrt(sample[0] / sample[1]) : 0.0,
+                          (double)sq / (double)std::max<int64_t>(h->inst_h[i].n, 1));
             h->inst_h[i].key_base = (uint32_t)keys;
             keys += (uint64_t)h->inst_h[i].M[0] * h->inst_h[i].M[1] * h->inst_h[i].M[2];
             if (keys >= (uint64_t)UINT32_MAX - 2 * (uint64_t)kScanTile)
                 return bail(fail(h, KMC_ERANGE, "search grid exceeds 2^32 keys; set sub_cells"));
         }
+        for (auto& I : h->inst_h) I.chi = h->filter_chi;
         h->n_keys = (uint32_t)keys;
         h->cbin_moments = 1;
         for (const InstDev& I : h->inst_h)
@@ -730,11 +781,29 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         h->any_direct = 0;
         int prune_any = 0;
         const bool dsmc = (h->cfg.flags & KMC_FLAG_DSMC) != 0;
+        // An option that asks for one of the other searches (speed only) takes the
+        // filtered one away from every instance: a flag, or tile parameters where a
+        // tile search would use them.
+        bool tile_grid = false;
+        for (const InstDev& I : h->inst_h) tile_grid = tile_grid || (I.s[0] == 1 && I.s[1] == 1 && I.s[2] == 1) || I.prune;
+        const bool choose = !dsmc && n > 0 &&
+                            !(h->cfg.flags & (KMC_FLAG_NO_TILE_SEARCH | KMC_FLAG_STAGED_SEARCH | KMC_FLAG_NO_TILE_PRUNE)) &&
+                            !(tile_grid && (h->cfg.tile_threads > 0 || h->cfg.tile_cap > 0 || h->cfg.tile_split > 0));
+        h->filtered = 0;
         for (auto& I : h->inst_h) {
             if (dsmc) {   // no closest-approach search at all
                 I.staged = I.tiled = 0;
                 continue;
             }
+            if (choose) {
+                I.tiled = 0;
+                I.prune = I.prune && I.n > 0;
+                h->filtered |= I.filtered;
+                h->any_direct |= I.n > 0 && !I.filtered;
+                prune_any |= I.prune;
+                continue;
+            }
+            I.filtered = 0;
             I.tiled = !I.staged && I.n > 0 && ((I.s[0] == 1 && I.s[1] == 1 && I.s[2] == 1) || I.prune) &&
                       !(h->cfg.flags & KMC_FLAG_NO_TILE_SEARCH);
             I.prune = I.prune && I.tiled;
@@ -744,6 +813,13 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
             prune_any |= I.prune;
         }
         h->tile_prune = prune_any;
+        if (h->filtered) {
+            int dev = 0, sms = 0;
+            if (cudaGetDevice(&dev) != cudaSuccess ||
+                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+                return bail(fail(h, KMC_ECUDA, "device attributes failed"));
+            h->filter_split = filter_split(n, sms);
+        }
         // the pruned search's default staging capacity fills 4 blocks per SM
         if (prune_any && h->cfg.tile_cap == 0 && !h->any_plain_tiled) h->tile_cap = kPrunedCap;
         if (cudaMemcpyAsync(h->inst_d, h->inst_h.data(), sizeof(InstDev) * h->n_inst, cudaMemcpyHostToDevice,
@@ -965,7 +1041,8 @@ int kmc_autotune(const kmc_config* cfg, int64_t n, const void* pos, const void* 
         // settings that end in an already timed set-up (same subdivision and
         // search kernel for every instance) are not timed again
         std::vector<int> setup;
-        for (const InstDev& I : h->inst_h) setup.insert(setup.end(), {I.s[0], I.s[1], I.s[2], I.tiled, I.staged});
+        for (const InstDev& I : h->inst_h)
+            setup.insert(setup.end(), {I.s[0], I.s[1], I.s[2], I.tiled, I.staged, I.filtered});
         setup.push_back(h->any_tiled ? h->tile_threads : 0);
         setup.push_back(h->any_tiled ? h->tile_cap : 0);
         setup.push_back(h->any_tiled ? h->tile_split : 0);
@@ -1043,7 +1120,7 @@ int kmc_get_info(kmc_handle* h, kmc_info* info) {
     // search, staged search, move, scan, two scatter passes,
     // then moments and two finalize kernels when moments are wanted
     info->kernels_per_step = ((h->any_direct || h->n_stage_tiles > 0) ? 1 : 0) + (h->any_plain_tiled ? 1 : 0) +
-                             (h->tile_prune ? 1 : 0) +
+                             (h->any_tiled && h->tile_prune ? 1 : 0) + (h->filtered ? 2 : 0) +   // operands, search
                              (h->n_stage_tiles > 0 ? 1 : 0) + ((h->cfg.flags & KMC_FLAG_DSMC) ? 1 : 0) + 4;
     info->kernels_moments = 3;
     info->tile_threads = h->tile_threads;

@@ -1,5 +1,5 @@
 // kmc_f64.cu -- binary64-state instantiation of the step kernels.
-#include "kmc_kernels.cuh"
+#include "kmc_filter.cuh"
 
 namespace kmc {
 KMC_INSTANTIATE(double)

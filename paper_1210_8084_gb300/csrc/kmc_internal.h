@@ -23,6 +23,8 @@ constexpr int kTestSlots = 256;        // counters of the pruned tile search's p
 constexpr int kCbinRows = 4;           // rows of search cells per c-bin up to which moments go one warp per c-bin
 constexpr int kPrunedCap = 1888;       // default staging capacity of the pruned tile search (28 B per slot)
                                        // count, Sum v.r_hat
+constexpr double kSymPassing = 64.0;   // filtered search: passing candidates per particle up to which a pair is tested once
+constexpr double kChiHits = 50.0;      // pairs per particle left by one filter from which it filters by criterion 1 too
 constexpr int kMomStride = 18;         // per c-bin output: 8 raw, 8 derived, Sum v.r_hat, v_r
 constexpr uint32_t kCanonMax = 16384;  // search cells up to this many particles are put in id order
 
@@ -54,6 +56,9 @@ struct InstDev {
     int staged;
     int tiled;           // search cells are the c-bins: one block per cell (tile_search_kernel)
     int prune;           // tiled, binary32: candidate clusters out of a warp's reach are skipped
+    int filtered;        // searched by the filtered search (kmc_filter.cuh), else one thread per particle
+    int chi;             // filtered search: criterion 1 filters too (the same for every instance of a handle)
+    int sym;             // filtered search, binary32: each pair tested once, by its lower position
     int adaptive;        // timestep dx_min / v_max(t) per step (Sect. "Simulation setup")
     double dx_min;       // smallest c-bin width over the position dimensions
     int tile_rows;
@@ -71,6 +76,18 @@ struct InstDyn {
     float dtf;                      // dt rounded to binary32
     int k[3];                       // search half-window in search cells
     int mom_e[3];                   // moment sums: fixed-point exponents of v, v^2 and W
+    // filtered search (kmc_filter.cuh): frames of 2^f_shift search cells (at most all), coordinates
+    // in units of 1 / f_scale (a power of two); f_box a length, the other
+    // margins in the square of those units (f_g1, f_c1 per unit of displacement)
+    int f_shift[3];
+    float f_w[3];                   // search cell widths (binary32)
+    int f_image;                    // a window may hold a pair at more than half a periodic box
+    float f_scale, f_sc2;           // scale, scale^2
+    float f_g0, f_g1;               // a particle's share of F's margin: f_g0 + f_g1 |s|
+    float f_c0, f_c1;               // the same of the margin of a and f
+    float f_thr;                    // threshold at the contact distance
+    float f_rt, f_slack;            // threshold at distance d: d^2 f_sc2 + f_rt d + f_slack
+    float f_box;                    // widening of a home's swept box
 };
 
 struct Geo {
@@ -145,6 +162,9 @@ struct Bufs {
     int any_direct;          // some instance uses the direct (per-thread) search
     int any_tiled;           // some instance uses the tile search (one block per c-bin)
     int any_plain_tiled;     // some tiled instance searches on its c-bins (not pruned)
+    int filtered;            // some instance is searched by the filtered search (kmc_filter.cuh)
+    int filter_chi;          // it also filters by criterion 1
+    int filter_split;        // log2 of the warps that share a group of 32 homes
     int dsmc;                // the random-partner comparison variant instead of the PoCA search
     int radial;              // accumulate Sum v.r_hat (KMC_FLAG_RADIAL_MOMENT)
     int cbin_moments;        // every c-bin is at most kCbinRows runs of search cells: moments per c-bin
@@ -167,6 +187,8 @@ template <typename T>
 cudaError_t launch_search(const Bufs<T>& b, cudaStream_t s);       // staged + per-particle search
 template <typename T>
 cudaError_t launch_tile_search(const Bufs<T>& b, cudaStream_t s);  // one block per c-bin (tiled instances)
+template <typename T>
+cudaError_t launch_filtered_search(const Bufs<T>& b, cudaStream_t s);  // tensor-core filter, every instance
 template <typename T>
 cudaError_t prepare_staged(const Bufs<T>& b);
 template <typename T>
@@ -192,7 +214,26 @@ cudaError_t launch_perm(const Bufs<T>& b, int32_t* perm, cudaStream_t s);
 template <typename T>
 cudaError_t launch_dsmc(const Bufs<T>& b, cudaStream_t s);     // random-partner collisions per c-bin
 template <typename T>
-cudaError_t launch_cbin_hist(const Bufs<T>& b, uint32_t* hist, unsigned long long* vmax2, cudaStream_t s);
+cudaError_t launch_cbin_hist(const Bufs<T>& b, uint32_t* hist, unsigned long long* vmax2, double* sample, cudaStream_t s);
+
+// log2 of the warps that share a group of 32 homes of the filtered search: a
+// small system has too few groups to fill the chip, so up to eight warps (a
+// block) take one group, until about 16 warps per SM are busy.
+inline int filter_split(int64_t n, int sms) {
+    const int64_t groups = (n + 31) / 32;
+    int s = 0;
+    while (s < 3 && (groups << s) < (int64_t)sms * 16) ++s;
+    return s;
+}
+
+// Whether the filtered search is the faster one for a particle with `cand`
+// candidates in its window, `hits` of which pass the filter (binary32).  Cost per
+// particle in ps, fitted to both searches on a GB300: one thread per particle 1.3
+// per candidate (16M slab tube 75 at 15, 2M-particle tubes 280 at 133 and 1730 at
+// 1489, 8M blast 265 at 213, 5M Noh 170 at 181); filtered 150 + 0.06 per
+// candidate + 5 per pair left (180 at 213 and 5; 590 at 181 and 90; 510 at 5282
+// and 13).
+inline bool filter_pays(double cand, double hits) { return 150.0 + 0.06 * cand + 5.0 * hits < 1.3 * cand; }
 
 // precision-independent
 cudaError_t launch_scan(uint32_t* count, uint32_t* start, uint32_t n_keys, uint32_t n_tiles,

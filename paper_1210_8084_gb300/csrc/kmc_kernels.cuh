@@ -823,7 +823,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) search_kerne
     const uint32_t tag = R<T>::bits(P.w);
     const int inst = tag_inst(b, tag);
     const InstDev& I = b.inst[inst];
-    if (I.tiled) return;   // searched, and its slot_of recorded, by the tile search
+    if (I.tiled || I.filtered) return;   // searched, and its slot_of recorded, by another kernel
     // sorted position by id, read by the move kernel to find a partner
     b.slot_of[I.p_off + (int64_t)tag_id(b, tag)] = (uint32_t)p;
     if (I.staged || absorbed(Q.w)) return;   // searched by the staged kernel, or gone
@@ -3056,11 +3056,14 @@ __global__ void __launch_bounds__(kThreads) window_count_kernel(Bufs<T> b, unsig
     if (lane_id() == 0 && cnt) atomicAdd(total, cnt);
 }
 
-// Particles per c-bin and largest |v|^2 per instance of the packed state in B
-// (statistics for the host's choice of search grid at init).
+// Particles per c-bin and largest |v|^2 per instance of the packed state in B, and
+// the sum of |v|^2 and the count of a sample (about a thousand blocks over the
+// whole state): statistics for the host's choice of search grid and search at
+// init.  The largest value is compared before the atomic (an atomic per warp on
+// one word took most of this kernel's time).
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads) cbin_hist_kernel(Bufs<T> b, uint32_t* __restrict__ hist,
-                                                             unsigned long long* vmax2) {
+                                                             unsigned long long* vmax2, double* sample) {
     using V = typename Vec4<T>::type;
     __shared__ GeoT<T> G;
     if (threadIdx.x == 0) G.load(b.geo);
@@ -3085,15 +3088,28 @@ __global__ void __launch_bounds__(kThreads) cbin_hist_kernel(Bufs<T> b, uint32_t
         if ((int)lane_id() == __ffs(peers) - 1) atomicAdd(hist + bin, (uint32_t)__popc(peers));
     }
     const double v2 = (double)Q.x * Q.x + (double)Q.y * Q.y + (double)Q.z * Q.z;
-    double m = live ? v2 : 0.0;
+    double m = live ? v2 : 0.0, t = m;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
+    for (int o = 16; o > 0; o >>= 1) {
+        m = fmax(m, __shfl_xor_sync(kFull, m, o));
+        t += __shfl_xor_sync(kFull, t, o);
+    }
     const int inst0 = __shfl_sync(kFull, inst, 0);
     const bool same = __all_sync(kFull, !valid || inst == inst0);
     if (same) {
-        if (lane_id() == 0 && valid) atomicMax(vmax2 + inst0, (unsigned long long)__double_as_longlong(m));
-    } else if (valid) {
+        const unsigned long long mb = (unsigned long long)__double_as_longlong(m);
+        const int cnt = __popc(__ballot_sync(kFull, live));
+        if (lane_id() == 0 && valid) {
+            if (mb > *((volatile unsigned long long*)(vmax2 + inst0))) atomicMax(vmax2 + inst0, mb);
+            if (blockIdx.x % ((gridDim.x + 1023u) / 1024u) == 0u) {
+                atomicAdd(sample + 2 * inst0, t);
+                atomicAdd(sample + 2 * inst0 + 1, (double)cnt);
+            }
+        }
+    } else if (live) {
         atomicMax(vmax2 + inst, (unsigned long long)__double_as_longlong(v2));
+        atomicAdd(sample + 2 * inst, v2);
+        atomicAdd(sample + 2 * inst + 1, 1.0);
     }
 }
 
@@ -3268,9 +3284,10 @@ cudaError_t launch_moments(const Bufs<T>& b, int use_virial, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t launch_cbin_hist(const Bufs<T>& b, uint32_t* hist, unsigned long long* vmax2, cudaStream_t s) {
+cudaError_t launch_cbin_hist(const Bufs<T>& b, uint32_t* hist, unsigned long long* vmax2, double* sample,
+                             cudaStream_t s) {
     if (b.n == 0) return cudaSuccess;
-    KMC_DIM_DISPATCH(b.geo.dim, cbin_hist_kernel, b, hist, vmax2);
+    KMC_DIM_DISPATCH(b.geo.dim, cbin_hist_kernel, b, hist, vmax2, sample);
     return cudaGetLastError();
 }
 
@@ -3295,7 +3312,8 @@ cudaError_t launch_window_count(const Bufs<T>& b, unsigned long long* total, cud
     template cudaError_t launch_gather_state<T>(const Bufs<T>&, T*, T*, cudaStream_t);             \
     template cudaError_t launch_cell_keys<T>(const Bufs<T>&, int32_t*, cudaStream_t);              \
     template cudaError_t launch_moments<T>(const Bufs<T>&, int, cudaStream_t);                     \
-    template cudaError_t launch_cbin_hist<T>(const Bufs<T>&, uint32_t*, unsigned long long*, cudaStream_t); \
+    template cudaError_t launch_filtered_search<T>(const Bufs<T>&, cudaStream_t);                  \
+    template cudaError_t launch_cbin_hist<T>(const Bufs<T>&, uint32_t*, unsigned long long*, double*, cudaStream_t); \
     template cudaError_t launch_window_count<T>(const Bufs<T>&, unsigned long long*, cudaStream_t);   \
     template cudaError_t launch_perm<T>(const Bufs<T>&, int32_t*, cudaStream_t);                   \
     template cudaError_t launch_dsmc<T>(const Bufs<T>&, cudaStream_t);

@@ -119,7 +119,19 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
         off += align256(bytes);
         return q;
     };
-    const size_t nv = (size_t)(n > 0 ? n : 1);
+    const size_t nv = ((size_t)(n > 0 ? n : 1) + 31) / 32 * 32;   // whole tiles of the filtered search
+    // The search as kmc_init chooses it (kmc_api.cu, choose_filter), without statistics
+    // of the state: mean density, windows of the contact distance and a search cell,
+    // each pair once unless many candidates lie within the contact distance.
+    double within = nbar, cand = nbar;
+    for (int d = 0; d < g.dim; ++d) {
+        within *= fmin(2.0 * sqrt(I.R2), fmin(3.0 * g.L[d] / g.n[d], g.L[d]));
+        const double k = ceil(sqrt(I.R2) / I.w[d]) + 1.0;   // search cells within the contact distance and a step
+        cand *= fmin((2.0 * k + 1.0) * I.w[d], fmin(3.0 * g.L[d] / g.n[d], g.L[d]));
+    }
+    I.sym = sizeof(T) == 4 && within <= 4.0 * kSymPassing ? 1 : 0;
+    I.filtered = sizeof(T) == 8 || filter_pays(cand, I.sym ? 0.25 * fmin(within, cand) : 0.05 * cand) ? 1 : 0;
+    I.chi = sizeof(T) == 8 ? 1 : 0;
     Bufs<T> b{};
     b.n = n;
     b.n_inst = 1;
@@ -143,9 +155,14 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     if (off > (size_t)KMC_STATIC_SCRATCH_BYTES) return KMC_ERANGE;
     b.n_keys = n_keys;
     b.n_tiles = n_tiles;
-    b.any_direct = 1;
-    b.tile_threads = 256;   // no instance here is tiled
-    b.tile_cap = 1536;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return KMC_ECUDA;
+    b.filtered = I.filtered;
+    b.any_direct = !I.filtered;
+    b.filter_chi = I.chi;
+    b.filter_split = filter_split(n, sms);
     b.id_bits = 32;
     b.id_mask = 0xffffffffu;
     // the array keeps the last call's contents: clear what must start at zero
@@ -162,7 +179,7 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     if (launch_scan(b.count, b.start, n_keys, n_tiles, b.scan_status, b.dyn, b.inst, 1, b.st, g, 0, s) != cudaSuccess)
         return KMC_ECUDA;
     if (launch_scatter<T>(b, s) != cudaSuccess) return KMC_ECUDA;
-    if (launch_search<T>(b, s) != cudaSuccess) return KMC_ECUDA;   // per particle (no instance is tiled here)
+    if ((I.filtered ? launch_filtered_search<T>(b, s) : launch_search<T>(b, s)) != cudaSuccess) return KMC_ECUDA;
     best_by_id<T><<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(b, best);
     return cudaGetLastError() == cudaSuccess ? KMC_OK : KMC_ECUDA;
 }

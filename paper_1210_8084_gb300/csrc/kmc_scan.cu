@@ -37,6 +37,75 @@ __device__ __forceinline__ int fixed_exponent(double m) {
     return e < -120 ? -120 : (e > 120 ? 120 : e);
 }
 
+// Frames, units and margins of the filtered search (derivation at the head of
+// kmc_filter.cuh) for a largest displacement s = v_max dt and a reach
+// D = R + 2 s.  The frames are as wide as keeps the rounding margin of an
+// ordinary pair to about a tenth of what decides it: R^2 + |v_rel|^2 dt^2 / 4
+// with one filter (R counts little where the threshold falls to the closest
+// candidate so far: R / 8), R and |v_rel| dt with three.  Every bound below holds
+// for any width.
+// Computed in binary32 (one thread per instance, in the way of the step; binary64
+// took 7 us): every bound carries a factor of 1 + 2^-10, far above its rounding.
+__device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo, float s, float D) {
+    const float up = 1.f + 0x1p-10f, r3 = 1.7320508f * up;
+    const float R2 = (float)in.R2 * (1.f + 0x1p-20f), Rc = sqrtf(R2) * (1.f + 0x1p-20f), Re = in.sym ? Rc : 0.125f * Rc;
+    s *= 1.f + 0x1p-20f;
+    D *= 1.f + 0x1p-20f;
+    float cmax = 0.f, lmax = 0.f, reach = 0.f;   // reach: largest separation of neighbouring c-bins, at most D
+    float w[3];
+    int image = 0;
+    for (int d = 0; d < geo.dim; ++d) {
+        w[d] = (float)in.w[d];
+        const float L = (float)geo.L[d];
+        cmax = fmaxf(cmax, fmaxf(fabsf((float)geo.lo[d]), fabsf((float)geo.hi[d])));
+        lmax = fmaxf(lmax, L);
+        reach = fmaxf(reach, fminf(D, 2.f * (float)in.s[d] * w[d]));
+        if (geo.bc[d] == KMC_BC_PERIODIC && (geo.n[d] < 5 || D >= 0.499f * L)) image = 1;
+    }
+    const float aim = in.chi ? fminf(200.f * Rc, 400.f * s) : 46.f * sqrtf(Re * Re + s * s / 16.f);
+    const float width = 2.f * (aim - reach - s);
+    float half = 0.f;
+    for (int d = 0; d < 3; ++d) {
+        int sh = 0;
+        dy.f_w[d] = 0.f;
+        if (d < geo.dim) {
+            while ((1 << sh) < in.M[d] && (float)min(2 << sh, in.M[d]) * w[d] <= width) ++sh;
+            half = fmaxf(half, 0.5f * (float)min(1 << sh, in.M[d]) * w[d]);
+            dy.f_w[d] = w[d];
+        }
+        dy.f_shift[d] = sh;
+    }
+    // largest coordinate of a candidate in its frame and of a home that may pair with it
+    const float X = (half + reach + s) * up;
+    const float sc = __int_as_float((127 + 4 - ilogbf(X)) << 23), sc2 = sc * sc;   // X sc in [16, 32)
+    const float e32 = 0x1p-20f * (cmax + lmax + s), tiny = 0x1p-23f / sc;
+    float slack = 0x1p-17f * D * D + 0x1p-18f * 12.f * X * X;
+    float E;   // error of a separation component that |r0| + |r1| (three filters) or |dm| (one) multiplies
+    if (in.chi) {
+        E = (0x1p-10f * X + e32 + tiny) * up;
+        const float Es = (0x1p-10f * s + 0x1p-20f * s + tiny) * up;   // of the displacements
+        dy.f_g0 = 1.5f * up * E * E * sc2;
+        dy.f_g1 = r3 * E * sc;
+        // criterion 1: a and f are off by at most sqrt(3) (E |s_rel| + Es |r|) + 3 E Es, |r| <= R + |s_i| + |s_j|
+        dy.f_c1 = r3 * (E + Es) * sc;
+        dy.f_c0 = ((0.5f * r3 * Rc * Es + 1.5f * E * Es) * up + (0x1p-19f * D + 0x1p-18f * 12.f * X) * s) * sc2;
+    } else {
+        E = (0x1p-21f * X + e32 + tiny) * up;
+        const float Eh = (0x1p-11f * s + 0x1p-20f * s + tiny) * up;   // of half displacements
+        slack += 0x1p-19f * X * X;   // the products of the low parts
+        dy.f_g0 = 1.5f * up * (E * E + Eh * Eh) * sc2;
+        dy.f_g1 = r3 * (E + Eh) * sc;
+        dy.f_c0 = dy.f_c1 = 0.f;
+    }
+    dy.f_image = image;
+    dy.f_scale = sc;
+    dy.f_sc2 = sc2;
+    dy.f_rt = 2.f * r3 * E * sc2;
+    dy.f_slack = slack * up * sc2;
+    dy.f_thr = (R2 + 2.f * r3 * E * Rc + slack * up) * sc2;
+    dy.f_box = Rc * up + 0x1p-9f * D + 0x1p-18f * (cmax + lmax);
+}
+
 __device__ void step_bookkeeping(InstDyn* dyn, const InstDev* inst, int n_inst, DevState* st, const Geo& geo,
                                  int bump) {
     for (int i = threadIdx.x; i < n_inst; i += blockDim.x) {
@@ -76,6 +145,7 @@ __device__ void step_bookkeeping(InstDyn* dyn, const InstDev* inst, int n_inst, 
         dyn[i].mom_e[1] = vm > 0.0 ? fixed_exponent(nn * vm * vm) : 120;
         const double wm = nn * 4.0 * sqrt(inst[i].R2) * vm;
         dyn[i].mom_e[2] = wm > 0.0 ? fixed_exponent(wm) : 120;
+        if (inst[i].filtered) filter_constants(dyn[i], inst[i], geo, (float)(vmax * dt), (float)D);
     }
     if (threadIdx.x == 0 && bump) st->step += 1u;
 }
