@@ -1121,7 +1121,8 @@ int kmc_get_info(kmc_handle* h, kmc_info* info) {
     // then moments and two finalize kernels when moments are wanted
     info->kernels_per_step = ((h->any_direct || h->n_stage_tiles > 0) ? 1 : 0) + (h->any_plain_tiled ? 1 : 0) +
                              (h->any_tiled && h->tile_prune ? 1 : 0) + (h->filtered ? 2 : 0) +   // operands, search
-                             (h->n_stage_tiles > 0 ? 1 : 0) + ((h->cfg.flags & KMC_FLAG_DSMC) ? 1 : 0) + 4;
+                             (h->n_stage_tiles > 0 ? 1 : 0) + ((h->cfg.flags & KMC_FLAG_DSMC) ? 1 : 0) +
+                             rank_launches(h->n, h->n_keys) + 4;
     info->kernels_moments = 3;
     info->tile_threads = h->tile_threads;
     info->tile_cap = h->tile_cap;

@@ -226,6 +226,17 @@ inline int filter_split(int64_t n, int sms) {
     return s;
 }
 
+// Counting-sort scatter of large cells (rank_cells_kernel): launches of it for a
+// state of n particles over n_keys search cells.
+constexpr uint32_t kRankMin = 64;        // cells up to this many particles: the moving pass counts
+constexpr int kRankCap = 4096;           // the first launch's largest cell (32 KiB of shared memory)
+constexpr int64_t kRankMean = 24;        // mean particles per cell from which the first launch runs
+constexpr int64_t kRankMeanLarge = 1024; // and from which the second runs, for cells up to kCanonMax
+inline int rank_launches(int64_t n, uint32_t n_keys) {
+    const int64_t mean = n_keys > 0 ? n / (int64_t)n_keys : 0;
+    return mean >= kRankMeanLarge ? 2 : mean >= kRankMean ? 1 : 0;
+}
+
 // Whether the filtered search is the faster one for a particle with `cand`
 // candidates in its window, `hits` of which pass the filter (binary32).  Cost per
 // particle in ps, fitted to both searches on a GB300: one thread per particle 1.3

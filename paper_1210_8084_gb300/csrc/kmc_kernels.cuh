@@ -2645,8 +2645,78 @@ __device__ __forceinline__ uint32_t tags_below(const uint32_t* __restrict__ t, u
     return r;
 }
 
+// Between the passes, where cells are large (rank_cap > 0): one block per cell of
+// kRankMin < N <= rank_cap particles replaces every tag by its rank in id order, so
+// that the moving pass reads a rank instead of counting the cell's tags (quadratic
+// in N).  The ids, spread over the instance's range, go to CAP / 2 buckets of
+// equal id range (a count, its prefix sums, a placement); a tag's rank is its
+// bucket's start plus the lower ids among the bucket's, about two for ids without
+// order (any order is right, a narrow range of ids only slower).  Both scatter
+// passes with this kernel, GB300: 64M particles in 262,144 cells (quadrants) 5.16 ->
+// 2.36 ms, 4M in 2000 cells 1.96 -> 0.12 ms.
+template <typename T, int CAP, int TPB>
+__global__ void __launch_bounds__(TPB) rank_cells_kernel(Bufs<T> b, uint32_t above) {
+    constexpr int NB = CAP / 2, PER = NB / TPB;
+    extern __shared__ uint32_t rank_smem[];
+    uint32_t* tg = rank_smem;                                                   // the cell's tags
+    uint32_t* cnt = tg + CAP;                                                   // buckets
+    unsigned short* idx = reinterpret_cast<unsigned short*>(cnt + NB);          // slots by bucket
+    __shared__ uint32_t wsum[TPB / 32];
+    const uint32_t kc = blockIdx.x;
+    const uint32_t s0 = b.start[kc], s1 = b.start[kc + 1];
+    const uint32_t N = s1 - s0;
+    if (s1 <= s0 || N <= above || N > (uint32_t)CAP || s1 > (uint32_t)b.n) return;   // block-uniform
+    int lo = 0, hi = b.n_inst - 1;   // instance of the cell (consecutive key ranges)
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (b.inst[mid].key_base <= kc) lo = mid;
+        else hi = mid - 1;
+    }
+    const float scale = (float)NB / (float)b.inst[lo].n;
+    auto bucket = [&](uint32_t tag) { return min(NB - 1, (int)((float)tag_id(b, tag) * scale)); };
+    uint32_t* tags = b.slot_of + s0;
+    const int t = threadIdx.x;
+    for (int i = t; i < NB; i += TPB) cnt[i] = 0u;
+    __syncthreads();
+    for (uint32_t i = t; i < N; i += TPB) {
+        const uint32_t tag = tags[i];
+        tg[i] = tag;
+        atomicAdd(&cnt[bucket(tag)], 1u);
+    }
+    __syncthreads();
+    uint32_t own[PER], sum = 0u;   // exclusive prefix sums of the counts
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        own[j] = sum;
+        sum += cnt[t * PER + j];
+    }
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, o);
+        if ((int)lane_id() >= o) inc += y;
+    }
+    if (lane_id() == 31) wsum[t >> 5] = inc;
+    __syncthreads();
+    uint32_t before = inc - sum;
+    for (int w = 0; w < (t >> 5); ++w) before += wsum[w];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) cnt[t * PER + j] = before + own[j];
+    __syncthreads();
+    for (uint32_t i = t; i < N; i += TPB) idx[atomicAdd(&cnt[bucket(tg[i])], 1u)] = (unsigned short)i;
+    __syncthreads();   // cnt[k] is now the end of bucket k
+    for (uint32_t i = t; i < N; i += TPB) {
+        const uint32_t tag = tg[i];
+        const int k = bucket(tag);
+        const uint32_t q0 = k > 0 ? cnt[k - 1] : 0u, q1 = cnt[k];
+        uint32_t r = q0;
+        for (uint32_t q = q0; q < q1; ++q) r += tg[idx[q]] < tag ? 1u : 0u;
+        tags[i] = r;
+    }
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kThreads, 8) scatter_kernel(Bufs<T> b) {
+__global__ void __launch_bounds__(kThreads, 8) scatter_kernel(Bufs<T> b, uint32_t rank_cap) {
     using V = typename Vec4<T>::type;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= b.n) return;
@@ -2656,7 +2726,11 @@ __global__ void __launch_bounds__(kThreads, 8) scatter_kernel(Bufs<T> b) {
     const uint32_t s0 = b.start[k];
     const uint32_t s1 = k < b.n_keys ? b.start[k + 1] : s0;
     uint32_t rank = slot;
-    if (s1 > s0 + 1u && s1 - s0 <= kCanonMax && s1 <= (uint32_t)b.n) rank = tags_below(b.slot_of, s0, s1, tag);
+    if (s1 > s0 + 1u && s1 - s0 <= kCanonMax && s1 <= (uint32_t)b.n) {
+        const uint32_t N = s1 - s0;
+        if (N > kRankMin && N <= rank_cap) rank = slot < N ? b.slot_of[s0 + slot] : slot;   // ranked already
+        else rank = tags_below(b.slot_of, s0, s1, tag);
+    }
     const uint32_t dst = s0 + rank;
     if (dst >= (uint32_t)b.n) {  // only after a failed scan; reported as a device error
         atomicOr(&b.st->error, kErrKeyRange);
@@ -3351,7 +3425,17 @@ cudaError_t launch_scatter(const Bufs<T>& b, cudaStream_t s) {
     if (b.n == 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((b.n + (int64_t)kThreads * kScatterItems - 1) / ((int64_t)kThreads * kScatterItems));
     scatter_tags_kernel<T><<<blocks, kThreads, 0, s>>>(b);
-    scatter_kernel<T><<<blocks_for(b.n), kThreads, 0, s>>>(b);
+    constexpr int kSmall = 256, kLarge = 1024;   // threads per block
+    const int large = (int)kCanonMax;
+    const int kernels = rank_launches(b.n, b.n_keys);
+    if (kernels > 0) rank_cells_kernel<T, kRankCap, kSmall><<<b.n_keys, kSmall, kRankCap * 8, s>>>(b, kRankMin);
+    if (kernels > 1) {
+        const cudaError_t e = cudaFuncSetAttribute(rank_cells_kernel<T, (int)kCanonMax, kLarge>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, large * 8);
+        if (e != cudaSuccess) return e;
+        rank_cells_kernel<T, (int)kCanonMax, kLarge><<<b.n_keys, kLarge, large * 8, s>>>(b, (uint32_t)kRankCap);
+    }
+    scatter_kernel<T><<<blocks_for(b.n), kThreads, 0, s>>>(b, kernels > 1 ? kCanonMax : kernels > 0 ? kRankCap : 0u);
     return cudaGetLastError();
 }
 

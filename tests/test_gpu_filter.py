@@ -45,17 +45,17 @@ def test_filtered_search_matches_oracle_and_per_particle_search(case):
         pos[:, 0] = np.where(pos[:, 0] >= hi[0], lo[0], pos[:, 0])
     dtype = np.float32 if prec == 32 else np.float64
     pos, vel = inputs.cast_state(pos, vel, dtype, lo, hi, bc)
-    out = []
+    out, kernels = [], []
     for flags in (0, k.KMC_FLAG_NO_TILE_SEARCH):
         sim = k.Simulation(k.make_config(dim_pos=dim, n_cells=cells, lo=lo, hi=hi, bc=bc, lam=lam, dt=dt, seed=3,
                                          precision=prec, flags=flags | k.KMC_FLAG_RECORD), pos, vel)
-        kernels = sim.info().kernels_per_step   # operands and search, or search; then four more
-        assert kernels == (6 if filtered and not flags else 5)
+        kernels.append(sim.info().kernels_per_step)
         sim.step(1)
         first = sim.partners()
         sim.step(2)
         out.append((first, sim.partners(), sim.state()))
         sim.close()
+    assert kernels[0] - kernels[1] == int(filtered)   # operands and search, or one search
     (f0, l0, s0), (f1, l1, s1) = out
     vol = np.prod([hi[d] - lo[d] for d in range(dim)])
     P = oracle.make_params(dim, cells, lo, hi, bc, R2=oracle.contact_R2(lam, 0.0, n / vol), dt=dt, seed=3, step=0,
