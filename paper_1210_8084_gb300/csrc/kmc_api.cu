@@ -974,14 +974,13 @@ int kmc_moments(kmc_handle* h, double* out, int where, int mask) {
     }
     const cudaMemcpyKind kind = where == KMC_WHERE_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     double* o = out;
+    const size_t rows8 = 8 * sizeof(double) * (size_t)h->n_bins;
     if (h->n_bins > 0 && (mask & KMC_MOM_RAW)) {
-        KMC_CUDA(h, cudaMemcpy2DAsync(o, 8 * sizeof(double), h->mom, kMomStride * sizeof(double), 8 * sizeof(double),
-                                      (size_t)h->n_bins, kind, h->stream));
+        KMC_CUDA(h, cudaMemcpyAsync(o, h->mom, rows8, kind, h->stream));
         o += 8 * h->n_bins;
     }
     if (h->n_bins > 0 && (mask & KMC_MOM_DERIVED)) {
-        KMC_CUDA(h, cudaMemcpy2DAsync(o, 8 * sizeof(double), h->mom + 8, kMomStride * sizeof(double), 8 * sizeof(double),
-                                      (size_t)h->n_bins, kind, h->stream));
+        KMC_CUDA(h, cudaMemcpyAsync(o, h->mom + 8 * h->n_bins, rows8, kind, h->stream));
         o += 8 * h->n_bins;
     }
     if (mask & KMC_MOM_GLOBAL) {
@@ -991,8 +990,7 @@ int kmc_moments(kmc_handle* h, double* out, int where, int mask) {
     if ((mask & KMC_MOM_RADIAL) && !(h->cfg.flags & KMC_FLAG_RADIAL_MOMENT))
         return fail(h, KMC_ESTATE, "KMC_MOM_RADIAL needs a handle created with KMC_FLAG_RADIAL_MOMENT");
     if (h->n_bins > 0 && (mask & KMC_MOM_RADIAL)) {
-        KMC_CUDA(h, cudaMemcpy2DAsync(o, 2 * sizeof(double), h->mom + 16, kMomStride * sizeof(double),
-                                      2 * sizeof(double), (size_t)h->n_bins, kind, h->stream));
+        KMC_CUDA(h, cudaMemcpyAsync(o, h->mom + 16 * h->n_bins, 2 * sizeof(double) * (size_t)h->n_bins, kind, h->stream));
     }
     if (where == KMC_WHERE_HOST) return check_device_error(h);
     return KMC_OK;

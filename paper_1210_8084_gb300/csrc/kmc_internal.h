@@ -25,7 +25,7 @@ constexpr int kPrunedCap = 1888;       // default staging capacity of the pruned
                                        // count, Sum v.r_hat
 constexpr double kSymPassing = 64.0;   // filtered search: passing candidates per particle up to which a pair is tested once
 constexpr double kChiHits = 50.0;      // pairs per particle left by one filter from which it filters by criterion 1 too
-constexpr int kMomStride = 18;         // per c-bin output: 8 raw, 8 derived, Sum v.r_hat, v_r
+constexpr int kMomStride = 18;         // per c-bin output: 8 raw, 8 derived, Sum v.r_hat and v_r (an array each)
 constexpr uint32_t kCanonMax = 16384;  // search cells up to this many particles are put in id order
 
 // device error flags (DevState::error)
@@ -147,7 +147,7 @@ struct Bufs {
     uint32_t n_keys;
     uint32_t n_tiles;
     unsigned long long* acc; // [n_bins * kAccFields] moment sums, fixed point (two's complement)
-    double* mom;             // [n_bins * kMomStride] raw, derived, radial
+    double* mom;             // raw [n_bins][8], derived [n_bins][8], radial [n_bins][2]
     double* glob;            // [n_inst * 8]
     int64_t n_bins;
     int32_t* rec_best;       // RECORD: [n] by global id

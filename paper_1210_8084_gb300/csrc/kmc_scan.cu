@@ -257,28 +257,55 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(uint32_t* __restrict
     }
 }
 
-// Fixed-point sum -> binary64 (exact below 2^53, correctly rounded above).
-__device__ __forceinline__ double unfix(unsigned long long a, int e) { return ldexp((double)(long long)a, -e); }
+// Fixed-point sum -> binary64 (exact below 2^53, correctly rounded above).  The
+// scaling by 2^-e, |e| <= 120, is an addition to the exponent: a non-zero sum
+// lies in [1, 2^63).  (ldexp took a dozen binary64 operations, which run at 1/64 of
+// the binary32 rate.)
+__device__ __forceinline__ double unfix(unsigned long long a, int e) {
+    const double x = (double)(long long)a;
+    return x == 0.0 ? 0.0 : __longlong_as_double(__double_as_longlong(x) - ((long long)e << 52));
+}
+
+// a / b from the correctly rounded reciprocal r of b: one Newton step on the
+// quotient, correctly rounded by Markstein's theorem (IBM J. Res. Dev. 34, 1990)
+// for operands away from the ends of the range, as here.
+__device__ __forceinline__ double div_rcp(double a, double b, double r) {
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+}
 
 // Derived per-c-bin moments (Eqs. vel_b, stress, 18, 19 with the readings
 // u = Sum v / N, v_rms^2 = <|v - u|^2>, T = v_rms^2 / 3, p = n T + virial),
 // and the per-instance integer totals of the fixed-point sums (exact, so the
-// order of the atomics does not matter): a warp whose bins belong to one
-// instance reduces with shuffles and adds once.
-__global__ void __launch_bounds__(256) finalize_bins_kernel(const InstDev* __restrict__ inst,
-                                                            const InstDyn* __restrict__ dyn, Geo geo,
-                                                            const unsigned long long* __restrict__ acc,
-                                                            double* __restrict__ mom, unsigned long long* gacc,
-                                                            int64_t n_bins, int64_t bins_per_inst) {
-    const int64_t bidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// order of the atomics does not matter): a block whose bins belong to one
+// instance adds once per total.  Bound by the binary64 operations; rows of the
+// result leave through shared memory as whole runs.  1,000,000 c-bins, GB300: 0.329 ms
+// with a division per quotient, ldexp, row-strided stores and seven atomics per
+// warp -> 0.111 ms.
+constexpr int kFinThreads = 128;
+__global__ void __launch_bounds__(kFinThreads) finalize_bins_kernel(const InstDev* __restrict__ inst,
+                                                                    const InstDyn* __restrict__ dyn, Geo geo,
+                                                                    const unsigned long long* __restrict__ acc,
+                                                                    double* __restrict__ mom, unsigned long long* gacc,
+                                                                    int64_t n_bins, int64_t bins_per_inst, double Vc) {
+    constexpr int kWarps = kFinThreads / 32;
+    __shared__ double out[kFinThreads][17];              // a row of 8 raw and 8 derived (17: no bank conflicts)
+    __shared__ unsigned long long part[kWarps][7];
+    const int64_t first = (int64_t)blockIdx.x * kFinThreads, bidx = first + threadIdx.x;
     const bool valid = bidx < n_bins;
     const int i = valid ? (int)(bidx / bins_per_inst) : 0;
+    const bool one = first / bins_per_inst == min(first + kFinThreads - 1, n_bins - 1) / bins_per_inst;   // block-uniform
     unsigned long long t[7] = {0, 0, 0, 0, 0, 0, 0};
     if (valid) {
         const InstDyn& D = dyn[i];
-        const unsigned long long* a = acc + bidx * kAccFields;
         unsigned long long ai[kAccFields];
-        for (int k = 0; k < kAccFields; ++k) ai[k] = a[k];
+        const ulonglong2* a2 = reinterpret_cast<const ulonglong2*>(acc + bidx * kAccFields);   // 80 bytes: aligned
+#pragma unroll
+        for (int k = 0; k < kAccFields / 2; ++k) {
+            const ulonglong2 v = a2[k];
+            ai[2 * k] = v.x;
+            ai[2 * k + 1] = v.y;
+        }
         t[0] = ai[0];
         t[1] = ai[4] + ai[5] + ai[6];
         t[2] = ai[1];
@@ -286,46 +313,54 @@ __global__ void __launch_bounds__(256) finalize_bins_kernel(const InstDev* __res
         t[4] = ai[3];
         t[5] = ai[7];
         t[6] = ai[8];
-        double* o = mom + bidx * kMomStride;
+        double* o = out[threadIdx.x];
         double r[8];
         r[0] = (double)(long long)ai[0];
         for (int k = 1; k <= 3; ++k) r[k] = unfix(ai[k], D.mom_e[0]);
         for (int k = 4; k <= 6; ++k) r[k] = unfix(ai[k], D.mom_e[1]);
         r[7] = unfix(ai[7], D.mom_e[2]);
         for (int k = 0; k < 8; ++k) o[k] = r[k];
-        double Vc = 1.0;
-        for (int d = 0; d < geo.dim; ++d) Vc *= geo.L[d] / (double)geo.n[d];
         const double N = r[0];
+        double vr = 0.0;
         const double svr = unfix(ai[9], D.mom_e[0]);
-        o[16] = svr;
-        o[17] = N > 0.0 ? svr / N : 0.0;   // Eq. vel_r
         if (N <= 0.0) {
             for (int k = 8; k < 16; ++k) o[k] = 0.0;
         } else {
             const double dt = D.dt_prev;   // the step whose collisions W sums
-            const double ux = r[1] / N, uy = r[2] / N, uz = r[3] / N;
-            const double c2 = (r[4] + r[5] + r[6]) / N - (ux * ux + uy * uy + uz * uz);
-            const double T = c2 / (geo.vdim == 2 ? 2.0 : 3.0);   // f velocity degrees of freedom
+            const double rN = __drcp_rn(N);
+            const double ux = div_rcp(r[1], N, rN), uy = div_rcp(r[2], N, rN), uz = div_rcp(r[3], N, rN);
+            const double c2 = div_rcp(r[4] + r[5] + r[6], N, rN) - (ux * ux + uy * uy + uz * uz);
+            // f velocity degrees of freedom
+            const double T = geo.vdim == 2 ? 0.5 * c2 : div_rcp(c2, 3.0, 1.0 / 3.0);
             const double nd = N / Vc;
             const double pkin = nd * T;
-            const double pvir = r[7] / (2.0 * geo.dim * Vc * dt);
+            const double pvir = r[7] == 0.0 ? 0.0 : r[7] / (2.0 * geo.dim * Vc * dt);
             o[8] = nd; o[9] = ux; o[10] = uy; o[11] = uz;
             o[12] = T; o[13] = pkin; o[14] = pvir; o[15] = pkin + pvir;
+            if (svr != 0.0) vr = div_rcp(svr, N, rN);   // Eq. vel_r
         }
+        *reinterpret_cast<double2*>(mom + 16 * n_bins + 2 * bidx) = make_double2(svr, vr);
     }
-    const int i0 = __shfl_sync(0xffffffffu, i, 0);
-    if (__all_sync(0xffffffffu, !valid || i == i0)) {
 #pragma unroll
-        for (int k = 0; k < 7; ++k) {
+    for (int k = 0; k < 7; ++k) {
+        if (one) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+            if ((threadIdx.x & 31u) == 0) part[threadIdx.x >> 5][k] = t[k];
+        } else if (valid && t[k]) {
+            atomicAdd(gacc + (size_t)i * 8 + k, t[k]);
         }
-        if ((threadIdx.x & 31u) == 0 && __shfl_sync(0xffffffffu, (int)valid, 0))
-            for (int k = 0; k < 7; ++k)
-                if (t[k]) atomicAdd(gacc + (size_t)i0 * 8 + k, t[k]);
-    } else if (valid) {
-        for (int k = 0; k < 7; ++k)
-            if (t[k]) atomicAdd(gacc + (size_t)i * 8 + k, t[k]);
+    }
+    __syncthreads();
+    if (one && threadIdx.x < 7) {
+        unsigned long long s = 0;
+        for (int w = 0; w < kWarps; ++w) s += part[w][threadIdx.x];
+        if (s) atomicAdd(gacc + (size_t)(first / bins_per_inst) * 8 + threadIdx.x, s);
+    }
+    const int words = 8 * (int)min((int64_t)kFinThreads, n_bins - first);
+    for (int w = threadIdx.x; w < words; w += kFinThreads) {
+        mom[8 * first + w] = out[w >> 3][w & 7];
+        mom[8 * (n_bins + first) + w] = out[w >> 3][8 + (w & 7)];
     }
 }
 
@@ -366,8 +401,10 @@ cudaError_t launch_finalize(const InstDev* inst, const InstDyn* dyn, int n_inst,
                             int64_t n_bins, cudaStream_t s) {
     if (n_bins == 0 || n_inst == 0) return cudaSuccess;
     const int64_t per = n_bins / n_inst;
-    finalize_bins_kernel<<<(unsigned)((n_bins + 255) / 256), 256, 0, s>>>(inst, dyn, geo, acc, mom, gacc, n_bins,
-                                                                         per);
+    double Vc = 1.0;
+    for (int d = 0; d < geo.dim; ++d) Vc *= geo.L[d] / (double)geo.n[d];
+    finalize_bins_kernel<<<(unsigned)((n_bins + kFinThreads - 1) / kFinThreads), kFinThreads, 0, s>>>(
+        inst, dyn, geo, acc, mom, gacc, n_bins, per, Vc);
     finalize_glob_kernel<<<(n_inst + 127) / 128, 128, 0, s>>>(dyn, gacc, glob, n_inst);
     return cudaGetLastError();
 }
