@@ -113,6 +113,7 @@ Bufs<T> make_bufs(const kmc_handle* h) {
     b.dyn = h->dyn_d;
     b.st = h->st_d;
     b.geo = h->geo;
+    b.g.load(h->geo);
     b.posA = (V*)h->posA;
     b.velA = (V*)h->velA;
     b.posB = (V*)h->posB;

@@ -44,7 +44,6 @@ namespace kmc {
 constexpr int kFiltTile = 8;      // candidates per tile (columns of one tensor instruction)
 constexpr int kFiltChunk = 4;     // tiles filtered at a time
 constexpr int kFiltList = 36;     // listed tiles: 3 left of a round and 32 of the next, a multiple of 4
-constexpr int kFiltWarps = 4;     // warps per block (8 where eight share a group)
 constexpr int kFiltQueue = 64;    // queued words of surviving pairs, one per lane and chunk (a power of two)
 constexpr int kFiltChunks = 32;   // chunks whose words may be queued or in test (a power of two)
 constexpr uint32_t kTilePart = 0x80000000u;   // listed tile that reaches past its row's range
@@ -150,9 +149,7 @@ __device__ __forceinline__ ChiTerms chi_terms(const float X[3], const float S[3]
 template <typename T, int DIM, bool CHI>
 __global__ void __launch_bounds__(kThreads) filter_prep_kernel(Bufs<T> b) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = p < b.n;
     float lo[3], hi[3];
@@ -359,10 +356,8 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
     using V = typename Vec4<T>::type;
     constexpr int F = DIM - 1;
     constexpr bool kF32 = sizeof(T) == 4;
-    __shared__ GeoT<T> G;
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     __shared__ FiltWarp<T> shared_warps[WARPS];
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FiltWarp<T>& W = shared_warps[warp];
     const int64_t group = ((int64_t)blockIdx.x * WARPS + warp) >> split;
@@ -878,11 +873,13 @@ template <typename T, int DIM, bool CHI>
 cudaError_t launch_filtered(const Bufs<T>& b, cudaStream_t s) {
     const int64_t warps = ((b.n + 31) / 32) << b.filter_split;
     filter_prep_kernel<T, DIM, CHI><<<blocks_for((b.n + 31) & ~(int64_t)31), kThreads, 0, s>>>(b);
-    if (b.filter_split == 3)
-        filter_search_kernel<T, DIM, CHI, 8><<<(unsigned)(warps / 8), 256, 0, s>>>(b, 3);
-    else
-        filter_search_kernel<T, DIM, CHI, kFiltWarps><<<(unsigned)((warps + kFiltWarps - 1) / kFiltWarps), kFiltWarps * 32,
-                                                        0, s>>>(b, b.filter_split);
+    // the warps that share a group are a block; a group of its own is a block of one
+    // warp (a block holds its place until its slowest warp is done: 4 warps took 8-10 %
+    // longer on the 3-D Sod tubes)
+    if (b.filter_split == 0) filter_search_kernel<T, DIM, CHI, 1><<<(unsigned)warps, 32, 0, s>>>(b, 0);
+    else if (b.filter_split < 3)
+        filter_search_kernel<T, DIM, CHI, 4><<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(b, b.filter_split);
+    else filter_search_kernel<T, DIM, CHI, 8><<<(unsigned)(warps / 8), 256, 0, s>>>(b, 3);
     return cudaGetLastError();
 }
 

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <string>
@@ -99,6 +100,32 @@ struct Geo {
     double rc[3];   // centre of the radial velocity moment
 };
 
+// The geometry in the state precision, a part of every kernel's parameters: its
+// values come from the constant bank.  For walled dimensions the half length is
+// +inf so the minimum-image shift never fires.
+template <typename T>
+struct GeoT {
+    T lo[3], hi[3], inv[3], L[3], hL[3], rc[3];
+    int n[3];
+    bool wall[3];     // no periodic wrap: reflective or absorbing
+    bool absorb[3];   // absorbing: a particle that ends a step outside is removed
+    int vdim;
+    void load(const Geo& g) {
+        vdim = g.vdim;
+        for (int d = 0; d < 3; ++d) {
+            lo[d] = (T)g.lo[d];
+            hi[d] = (T)g.hi[d];
+            inv[d] = (T)g.inv_dx[d];
+            L[d] = (T)g.L[d];
+            wall[d] = g.bc[d] != 0;
+            absorb[d] = g.bc[d] == 2;
+            hL[d] = wall[d] ? (T)INFINITY : (T)0.5 * L[d];
+            rc[d] = (T)g.rc[d];
+            n[d] = g.n[d];
+        }
+    }
+};
+
 struct DevState {
     uint32_t step;        // Philox counter word 1 of the step being taken
     uint32_t error;       // kErr* bits
@@ -133,6 +160,7 @@ struct Bufs {
     InstDyn* dyn;            // [n_inst]
     DevState* st;
     Geo geo;
+    GeoT<T> g;
     V* posA; V* velA;        // sorted state (search-grid key order)
     V* posB; V* velB;        // staging / unsorted end-of-step state
     unsigned long long* bkey;  // [n] partner key of A[p] (tag of the closest candidate, kNoPartner)

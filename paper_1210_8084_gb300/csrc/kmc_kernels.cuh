@@ -108,32 +108,6 @@ __device__ __forceinline__ void sincos_2pi(float u, float* s, float* c) { sincos
 __device__ __forceinline__ void sincos_2pi(double u, double* s, double* c) { sincospi(2.0 * u, s, c); }
 
 // ------------------------------------------------------------- geometry
-// Per-dimension constants in the state precision.  For walled dimensions the
-// half length is +inf so the minimum-image shift never fires.
-template <typename T>
-struct GeoT {
-    T lo[3], hi[3], inv[3], L[3], hL[3], rc[3];
-    int n[3];
-    bool wall[3];     // no periodic wrap: reflective or absorbing
-    bool absorb[3];   // absorbing: a particle that ends a step outside is removed
-    int vdim;
-    __device__ __forceinline__ void load(const Geo& g) {
-        vdim = g.vdim;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            lo[d] = (T)g.lo[d];
-            hi[d] = (T)g.hi[d];
-            inv[d] = (T)g.inv_dx[d];
-            L[d] = (T)g.L[d];
-            wall[d] = g.bc[d] != 0;
-            absorb[d] = g.bc[d] == 2;
-            hL[d] = wall[d] ? R<T>::inf() : (T)0.5 * L[d];
-            rc[d] = (T)g.rc[d];
-            n[d] = g.n[d];
-        }
-    }
-};
-
 // c-bin index c = floor((x - lo) * n / (hi - lo)) clamped to [0, n-1], and the
 // search cell g = c * s + floor(frac * s) inside it.
 template <typename T>
@@ -413,9 +387,7 @@ __global__ void __launch_bounds__(kThreads) pack_kernel(Bufs<T> b, const T* __re
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads) bin_kernel(Bufs<T> b) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = p < b.n;
     V P = {}, Q = {};
@@ -812,10 +784,8 @@ template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) search_kernel(Bufs<T> b) {
     using V = typename Vec4<T>::type;
     constexpr bool kSym = sizeof(T) == 4;
-    __shared__ GeoT<T> G;
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     __shared__ int2 rng[(DIM == 3 ? 9 : 3) * kThreads];
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= b.n) return;
     const V P = b.posA[p];
@@ -1976,7 +1946,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) tile_pruned_kernel(Bufs<float
     __shared__ GeoT<float> G;
     __shared__ int inst_s, c_s[3];
     if (threadIdx.x == 0) {
-        G.load(b.geo);
+        G = b.g;
         int c[3];
         inst_s = cbin_of_block<DIM>(b, b.geo, blockIdx.x, c);
         c_s[0] = c[0];
@@ -2006,7 +1976,7 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? 4 : 1) tile_sea
     __shared__ int64_t h0_s, h1_s;
     const uint32_t bc = blockIdx.x;
     if (threadIdx.x == 0) {
-        G.load(b.geo);
+        G = b.g;
         // instance of the c-bin (instances own consecutive c-bin ranges)
         int lo = 0, hi = b.n_inst - 1;
         while (lo < hi) {
@@ -2268,7 +2238,7 @@ __global__ void __launch_bounds__(kStageThreads) search_staged_kernel(Bufs<T> b)
     const int tid = threadIdx.x;
     const uint32_t tile = blockIdx.x;
     if (tid == 0) {
-        G.load(b.geo);
+        G = b.g;
         int lo = 0, hi = b.n_inst - 1;   // last instance with tile_base <= tile
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -2442,9 +2412,7 @@ __global__ void __launch_bounds__(kStageThreads) search_staged_kernel(Bufs<T> b)
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 8 : 1) move_kernel(Bufs<T> b) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = p < b.n;
     V P = {}, Q = {};
@@ -3042,9 +3010,7 @@ __global__ void __launch_bounds__(kThreads) fetch_kernel(Bufs<T> b, T* __restric
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads) cellkey_kernel(Bufs<T> b, int32_t* __restrict__ keys) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= b.n) return;
     const V P = b.posA[p];
@@ -3065,12 +3031,9 @@ __global__ void __launch_bounds__(kThreads) cellkey_kernel(Bufs<T> b, int32_t* _
 template <typename T, int DIM, bool RADIAL>
 __global__ void __launch_bounds__(kThreads) moments_kernel(Bufs<T> b, int use_virial) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     __shared__ MomentSlots S;
-    if (threadIdx.x == 0) {
-        G.load(b.geo);
-        S.n = 0;
-    }
+    if (threadIdx.x == 0) S.n = 0;
     __syncthreads();
     const int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kMomItems;
     uint32_t cur = 0xffffffffu;
@@ -3153,9 +3116,7 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(Bufs<T> b, int use_vi
 template <typename T, int DIM, bool RADIAL, int LANES>
 __global__ void __launch_bounds__(kThreads) moments_cbin_kernel(Bufs<T> b, int use_virial) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     const int64_t bin = (int64_t)blockIdx.x * (kThreads / LANES) + threadIdx.x / LANES;
     const bool live = bin < b.n_bins;
     const int64_t bc = live ? bin : b.n_bins - 1;   // lanes past the end follow the last c-bin and store nothing
@@ -3268,9 +3229,7 @@ __global__ void __launch_bounds__(kThreads) moments_cbin_kernel(Bufs<T> b, int u
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads) window_count_kernel(Bufs<T> b, unsigned long long* total) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long cnt = 0;
     if (p < b.n && !absorbed(b.velA[p].w)) {
@@ -3316,9 +3275,7 @@ template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads) cbin_hist_kernel(Bufs<T> b, uint32_t* __restrict__ hist,
                                                              unsigned long long* vmax2, double* sample) {
     using V = typename Vec4<T>::type;
-    __shared__ GeoT<T> G;
-    if (threadIdx.x == 0) G.load(b.geo);
-    __syncthreads();
+    const GeoT<T>& G = b.g;   // kernel parameter: constant bank
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = p < b.n;
     V P = {}, Q = {};

@@ -140,6 +140,7 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     b.dyn = (InstDyn*)take(sizeof(InstDyn));
     uint32_t* bad = (uint32_t*)take(sizeof(uint32_t));
     b.geo = g;
+    b.g.load(g);
     b.posA = (V*)take(nv * sizeof(V));
     b.velA = (V*)take(nv * sizeof(V));
     b.posB = (V*)take(nv * sizeof(V));
