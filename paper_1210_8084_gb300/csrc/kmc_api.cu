@@ -56,7 +56,7 @@ struct kmc_handle {
     uint32_t n_stage_tiles = 0;
     int stage_cap = 0, stage_rows = 0, stage_stride = 0, stage_pair_cap = 0, any_direct = 1, any_tiled = 0;
     int any_plain_tiled = 0;
-    int filtered = 0, filter_chi = 0, filter_split = 0;   // filtered search (see Bufs)
+    int filtered = 0, paired = 0, filter_chi = 0, filter_split = 0;   // filtered search (see Bufs)
     int cbin_moments = 0;   // moments one warp per c-bin (every c-bin: at most kCbinRows runs of search cells)
     int tile_threads = 256, tile_cap = 1536, tile_split = 1, tile_prune = 1;
     int64_t n_bins = 0, bins_per_inst = 0;
@@ -144,6 +144,7 @@ Bufs<T> make_bufs(const kmc_handle* h) {
     b.any_tiled = h->any_tiled;
     b.any_plain_tiled = h->any_plain_tiled;
     b.filtered = h->filtered;
+    b.paired = h->paired;
     b.filter_chi = h->filter_chi;
     b.filter_split = h->filter_split;
     b.dsmc = (h->cfg.flags & KMC_FLAG_DSMC) ? 1 : 0;
@@ -174,6 +175,7 @@ cudaError_t enqueue_step(kmc_handle* h, int want_moments, cudaEvent_t* ev = null
     } else {
         if ((e = launch_search<T>(b, s)) != cudaSuccess) return e;
         if (b.filtered && (e = launch_filtered_search<T>(b, s)) != cudaSuccess) return e;
+        if (b.paired && (e = launch_pairs_search<T>(b, s)) != cudaSuccess) return e;
     }
     if ((e = mark(KMC_PHASE_TILE)) != cudaSuccess) return e;
     if (!b.dsmc && (e = launch_tile_search<T>(b, s)) != cudaSuccess) return e;
@@ -343,19 +345,18 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
     }
 }
 
-// Search of instance i where no option asks for a particular one: the filtered
-// search or one thread per particle, and the filtered search's form.  Estimates
-// per particle: `occ` is the particles' mean occupancy of their c-bin; `cand`
+// Costs of an instance's searches where no option asks for a particular one, and the
+// forms of the filtered and the pair search.  Estimates per particle: `occ` is the particles' mean occupancy of their c-bin; `cand`
 // the candidates of the first step's window, `within` those inside the contact
 // distance (cut at the window), `passing` those that meet within an rms
 // displacement; `near` those one filter leaves (inside R and half a relative
 // displacement, about 1.1 vrms dt).
-// Binary32 looks at each pair once, its threshold then staying R^2, or, where many
-// candidates pass, at every home's whole window with a threshold that falls to
-// its closest candidate: twice the pairs, but few of them left (a twentieth on
-// the quadrant workload).  Binary64 always filters (its exact test runs at 1/64
+// The binary32 filter looks at each pair once, its threshold then staying R^2, or,
+// where many candidates pass, at every home's whole window with a threshold that
+// falls to its closest candidate: twice the pairs, but few of them left (a tenth
+// at 150-270 particles per c-bin of the quadrant workload).  Binary64 always filters (its exact test runs at 1/64
 // of the binary32 rate), by criterion 1 too.
-void choose_filter(kmc_handle* h, InstDev& I, double vmax, double vrms, double occ) {
+SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms, double occ) {
     const double dt0 = (I.adaptive && vmax > 0.0) ? I.dx_min / vmax : I.dt;
     const double R = sqrt(I.R2), reach = 1.001 * (R + 2.0 * vmax * dt0), rho = sqrt(I.R2 + 1.2 * vrms * vrms * dt0 * dt0);
     double cand = occ, within = occ, near = occ;
@@ -369,13 +370,57 @@ void choose_filter(kmc_handle* h, InstDev& I, double vmax, double vrms, double o
     const double passing = within * (R > 0.0 ? std::min(1.0, vrms * dt0 / R) : 0.0);
     I.sym = h->precision == 32 && passing <= kSymPassing ? 1 : 0;
     // a ball in the cube of near; each pair once
-    double hits = I.sym ? 0.5 * near * (h->dim == 3 ? 0.52 : 0.79) : 0.05 * cand;
+    double hits = I.sym ? 0.5 * near * (h->dim == 3 ? 0.52 : 0.79) : 0.1 * cand;
     if (I.sym && hits > kChiHits && R > 1.5 * vrms * dt0 && vmax < 6.0 * vrms) {
         h->filter_chi = 1;   // criterion 1 leaves about the passing ones
         hits = std::min(hits, 4.0 * passing);
     }
     if (h->precision == 64) h->filter_chi = 1;
-    I.filtered = I.n > 0 && (h->precision == 64 || I.prune || filter_pays(cand, hits)) ? 1 : 0;
+    double rows = 1.0, n_row = occ * h->geo.n[h->dim - 1];
+    for (int d = 0; d + 1 < h->dim; ++d) {
+        const double k = ceil((reach + 1e-5 * h->geo.L[d]) / I.w[d]);
+        rows *= std::min(2.0 * k + 1.0, (double)std::min(3 * I.s[d], I.M[d]));
+        n_row /= I.s[d];
+    }
+    I.close = passing > kPairsClose ? 1 : 0;
+    return search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, cand, hits, passing, rows, n_row);
+}
+
+// The searches of a handle's instances: pruned ones and binary64 are filtered, the
+// others by the set of searches that costs least.  A further search reads every
+// particle once more (6 ps each: a 158M-particle ensemble took 30.0 ms with the three
+// cheapest per instance and 27.9 ms with one).  A handle with pruned instances uses
+// no pair search.
+void choose_searches(kmc_handle* h, const std::vector<SearchCosts>& cost) {
+    bool prune = false;
+    int64_t n = 0;
+    for (const InstDev& I : h->inst_h) {
+        prune = prune || (I.prune && I.n > 0);
+        n += I.n;
+    }
+    unsigned best = 1u << kSearchFilter;
+    double least = INFINITY;
+    for (unsigned set = 1; set < 8 && h->precision == 32; ++set) {
+        if (prune && (set & (1u << kSearchPairs))) continue;
+        double sum = 0.0;
+        unsigned used = prune ? 1u << kSearchFilter : 0u;
+        for (int i = 0; i < h->n_inst; ++i) {
+            const InstDev& I = h->inst_h[i];
+            if (I.n == 0 || I.prune) continue;
+            const int k = cheapest_search(cost[i], set);
+            sum += (double)I.n * cost[i].ps[k];
+            used |= 1u << k;
+        }
+        for (int k = 0; k < 3; ++k) sum += (used >> k & 1u) ? 6.0 * (double)n : 0.0;
+        if (sum < least) {
+            least = sum;
+            best = set;
+        }
+    }
+    for (int i = 0; i < h->n_inst; ++i) {
+        InstDev& I = h->inst_h[i];
+        I.search = I.n == 0 ? kSearchDirect : I.prune ? kSearchFilter : cheapest_search(cost[i], best);
+    }
 }
 
 // Staged search plan (3-D only): a tile is tile_rows y-rows of one x-slab,
@@ -747,6 +792,8 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         if (!okc) return bail(fail(h, KMC_ECUDA, "search-grid statistics failed"));
         uint64_t keys = 0;
         std::vector<uint32_t> max_occ(h->n_inst, 0u);
+        std::vector<double> vmax(h->n_inst, 0.0), occ(h->n_inst, 0.0);
+        std::vector<SearchCosts> costs;
         for (int i = 0; i < h->n_inst; ++i) {
             uint32_t mx = 0;
             uint64_t sq = 0;   // of the occupancies
@@ -759,15 +806,19 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
             double v2;
             memcpy(&v2, &vm_h[i], sizeof(double));
             choose_subdivision(h, h->inst_h[i], sqrt(v2), mx);
-            double sample[2];
-            memcpy(sample, &vm_h[(size_t)h->n_inst + 2 * i], sizeof(sample));
-            choose_filter(h, h->inst_h[i], sqrt(v2), sample[1] > 0.0 ? sqrt(sample[0] / sample[1]) : 0.0,
-                          (double)sq / (double)std::max<int64_t>(h->inst_h[i].n, 1));
+            vmax[i] = sqrt(v2);
+            occ[i] = (double)sq / (double)std::max<int64_t>(h->inst_h[i].n, 1);
             h->inst_h[i].key_base = (uint32_t)keys;
             keys += (uint64_t)h->inst_h[i].M[0] * h->inst_h[i].M[1] * h->inst_h[i].M[2];
             if (keys >= (uint64_t)UINT32_MAX - 2 * (uint64_t)kScanTile)
                 return bail(fail(h, KMC_ERANGE, "search grid exceeds 2^32 keys; set sub_cells"));
         }
+        for (int i = 0; i < h->n_inst; ++i) {
+            double sample[2];
+            memcpy(sample, &vm_h[(size_t)h->n_inst + 2 * i], sizeof(sample));
+            costs.push_back(estimate_search(h, h->inst_h[i], vmax[i], sample[1] > 0.0 ? sqrt(sample[0] / sample[1]) : 0.0, occ[i]));
+        }
+        choose_searches(h, costs);
         for (auto& I : h->inst_h) I.chi = h->filter_chi;
         h->n_keys = (uint32_t)keys;
         h->cbin_moments = 1;
@@ -790,7 +841,8 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         const bool choose = !dsmc && n > 0 &&
                             !(h->cfg.flags & (KMC_FLAG_NO_TILE_SEARCH | KMC_FLAG_STAGED_SEARCH | KMC_FLAG_NO_TILE_PRUNE)) &&
                             !(tile_grid && (h->cfg.tile_threads > 0 || h->cfg.tile_cap > 0 || h->cfg.tile_split > 0));
-        h->filtered = 0;
+        h->filtered = h->paired = 0;
+        int64_t open = 0, close = 0;   // particles of pair-searched instances
         for (auto& I : h->inst_h) {
             if (dsmc) {   // no closest-approach search at all
                 I.staged = I.tiled = 0;
@@ -799,12 +851,13 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
             if (choose) {
                 I.tiled = 0;
                 I.prune = I.prune && I.n > 0;
-                h->filtered |= I.filtered;
-                h->any_direct |= I.n > 0 && !I.filtered;
+                h->filtered |= I.search == kSearchFilter;
+                if (I.search == kSearchPairs) (I.close ? close : open) += I.n;
+                h->any_direct |= I.n > 0 && I.search == kSearchDirect;
                 prune_any |= I.prune;
                 continue;
             }
-            I.filtered = 0;
+            I.search = kSearchDirect;
             I.tiled = !I.staged && I.n > 0 && ((I.s[0] == 1 && I.s[1] == 1 && I.s[2] == 1) || I.prune) &&
                       !(h->cfg.flags & KMC_FLAG_NO_TILE_SEARCH);
             I.prune = I.prune && I.tiled;
@@ -813,6 +866,7 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
             h->any_direct |= !I.tiled && !I.staged;   // searched one thread per particle
             prune_any |= I.prune;
         }
+        if (open + close > 0) h->paired = close > open ? 3 : 1;   // one form for the handle
         h->tile_prune = prune_any;
         if (h->filtered) {
             int dev = 0, sms = 0;
@@ -1041,7 +1095,7 @@ int kmc_autotune(const kmc_config* cfg, int64_t n, const void* pos, const void* 
         // search kernel for every instance) are not timed again
         std::vector<int> setup;
         for (const InstDev& I : h->inst_h)
-            setup.insert(setup.end(), {I.s[0], I.s[1], I.s[2], I.tiled, I.staged, I.filtered});
+            setup.insert(setup.end(), {I.s[0], I.s[1], I.s[2], I.tiled, I.staged, I.search});
         setup.push_back(h->any_tiled ? h->tile_threads : 0);
         setup.push_back(h->any_tiled ? h->tile_cap : 0);
         setup.push_back(h->any_tiled ? h->tile_split : 0);
@@ -1119,7 +1173,7 @@ int kmc_get_info(kmc_handle* h, kmc_info* info) {
     // search, staged search, move, scan, two scatter passes,
     // then moments and two finalize kernels when moments are wanted
     info->kernels_per_step = ((h->any_direct || h->n_stage_tiles > 0) ? 1 : 0) + (h->any_plain_tiled ? 1 : 0) +
-                             (h->any_tiled && h->tile_prune ? 1 : 0) + (h->filtered ? 2 : 0) +   // operands, search
+                             (h->any_tiled && h->tile_prune ? 1 : 0) + (h->filtered ? 2 : 0) + (h->paired ? 1 : 0) +   // operands and search
                              (h->n_stage_tiles > 0 ? 1 : 0) + ((h->cfg.flags & KMC_FLAG_DSMC) ? 1 : 0) +
                              rank_launches(h->n, h->n_keys) + 4;
     info->kernels_moments = 3;

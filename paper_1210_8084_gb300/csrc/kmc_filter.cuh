@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kThreads) filter_prep_kernel(Bufs<T> b) {
     }
     const InstDev& I = b.inst[inst];
     const InstDyn& D = b.dyn[inst];
-    if (valid && I.filtered) {
+    if (valid && I.search == kSearchFilter) {
         const uint32_t tag = R<T>::bits(P.w);
         // sorted position by id, read by the move kernel to find a partner
         b.slot_of[I.p_off + (int64_t)tag_id(b, tag)] = (uint32_t)p;
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
         W.vel[lane] = Q;
         inst = valid ? tag_inst(b, R<T>::bits(P.w)) : 0;
         const InstDev& I = b.inst[inst];
-        valid = valid && I.filtered;
+        valid = valid && I.search == kSearchFilter;
         int c, g0, g1 = 0;
         cell_and_search<T>(P.x, G.lo[0], G.inv[0], G.n[0], I.s[0], c, g0);
         if (DIM == 3) cell_and_search<T>(P.y, G.lo[1], G.inv[1], G.n[1], I.s[1], c, g1);

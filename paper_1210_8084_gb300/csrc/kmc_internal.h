@@ -25,6 +25,8 @@ constexpr int kCbinRows = 4;           // rows of search cells per c-bin up to w
 constexpr int kPrunedCap = 1888;       // default staging capacity of the pruned tile search (28 B per slot)
                                        // count, Sum v.r_hat
 constexpr double kSymPassing = 64.0;   // filtered search: passing candidates per particle up to which a pair is tested once
+constexpr double kPairsClose = 16.0;   // pair search: passing candidates per particle from which pairs are tested
+                                       // against the closest so far
 constexpr double kChiHits = 50.0;      // pairs per particle left by one filter from which it filters by criterion 1 too
 constexpr int kMomStride = 18;         // per c-bin output: 8 raw, 8 derived, Sum v.r_hat and v_r (an array each)
 constexpr uint32_t kCanonMax = 16384;  // search cells up to this many particles are put in id order
@@ -34,6 +36,10 @@ constexpr uint32_t kErrScanTimeout = 1u;
 constexpr uint32_t kErrKeyRange = 2u;
 
 constexpr unsigned long long kNoPartner = ~0ull;  // partner key of a particle without candidate
+// searches that no option asks for (InstDev::search)
+constexpr int kSearchDirect = 0;       // one thread per particle
+constexpr int kSearchFilter = 1;       // kmc_filter.cuh
+constexpr int kSearchPairs = 2;        // kmc_pairs.cuh, binary32
 constexpr int kMomItems = 4;           // moments: consecutive particles per thread
 constexpr int kStageThreads = 256;     // staged search: threads per tile
 
@@ -57,9 +63,10 @@ struct InstDev {
     int staged;
     int tiled;           // search cells are the c-bins: one block per cell (tile_search_kernel)
     int prune;           // tiled, binary32: candidate clusters out of a warp's reach are skipped
-    int filtered;        // searched by the filtered search (kmc_filter.cuh), else one thread per particle
+    int search;          // kSearch...: its search, unless tiled or staged
     int chi;             // filtered search: criterion 1 filters too (the same for every instance of a handle)
     int sym;             // filtered search, binary32: each pair tested once, by its lower position
+    int close;           // pair search: many candidates pass, pairs are tested against the closest so far
     int adaptive;        // timestep dx_min / v_max(t) per step (Sect. "Simulation setup")
     double dx_min;       // smallest c-bin width over the position dimensions
     int tile_rows;
@@ -89,6 +96,9 @@ struct InstDyn {
     float f_thr;                    // threshold at the contact distance
     float f_rt, f_slack;            // threshold at distance d: d^2 f_sc2 + f_rt d + f_slack
     float f_box;                    // widening of a home's swept box
+    // pair search (kmc_pairs.cuh)
+    int p_image;                    // a pair may meet at half a periodic box or more
+    float p_slack;                  // rounding of a squared distance of closest approach, in the test against the closest so far
 };
 
 struct Geo {
@@ -191,6 +201,8 @@ struct Bufs {
     int any_tiled;           // some instance uses the tile search (one block per c-bin)
     int any_plain_tiled;     // some tiled instance searches on its c-bins (not pruned)
     int filtered;            // some instance is searched by the filtered search (kmc_filter.cuh)
+    int paired;              // some instance is searched by lanes of homes against pairs (kmc_pairs.cuh): 1, or 3
+                             // where many candidates pass
     int filter_chi;          // it also filters by criterion 1
     int filter_split;        // log2 of the warps that share a group of 32 homes
     int dsmc;                // the random-partner comparison variant instead of the PoCA search
@@ -215,6 +227,8 @@ template <typename T>
 cudaError_t launch_search(const Bufs<T>& b, cudaStream_t s);       // staged + per-particle search
 template <typename T>
 cudaError_t launch_tile_search(const Bufs<T>& b, cudaStream_t s);  // one block per c-bin (tiled instances)
+template <typename T>
+cudaError_t launch_pairs_search(const Bufs<T>& b, cudaStream_t s);     // lanes of homes, pairs of candidates
 template <typename T>
 cudaError_t launch_filtered_search(const Bufs<T>& b, cudaStream_t s);  // tensor-core filter, every instance
 template <typename T>
@@ -265,14 +279,39 @@ inline int rank_launches(int64_t n, uint32_t n_keys) {
     return mean >= kRankMeanLarge ? 2 : mean >= kRankMean ? 1 : 0;
 }
 
-// Whether the filtered search is the faster one for a particle with `cand`
-// candidates in its window, `hits` of which pass the filter (binary32).  Cost per
-// particle in ps, fitted to both searches on a GB300: one thread per particle 1.3
-// per candidate (16M slab tube 75 at 15, 2M-particle tubes 280 at 133 and 1730 at
-// 1489, 8M blast 265 at 213, 5M Noh 170 at 181); filtered 150 + 0.06 per
-// candidate + 5 per pair left (180 at 213 and 5; 590 at 181 and 90; 510 at 5282
-// and 13).
-inline bool filter_pays(double cand, double hits) { return 150.0 + 0.06 * cand + 5.0 * hits < 1.3 * cand; }
+// Estimated costs of the three searches of a binary32 instance in ps per particle,
+// fitted on a GB300 to 36 states (slab tubes of 0.3M-16M particles with R from one to
+// sixty c-bins, 2-D implosions and quadrants, 3-D blasts).  `cand`: candidates in
+// a particle's window; `hits`: those that pass the filter; `passing`: those that meet;
+// `rows`: rows of search cells in the window; `n_row`: particles in a row of cells.
+// Measured / estimated, one thread per particle, filtered, pairs:
+//   16M slab tube, 14 candidates    70 / 88     - / 191    161 / 178
+//   4M slab, 206                   370 / 338  287 / 273    238 / 214
+//   4M slab, 469                   623 / 680  232 / 222    321 / 299
+//   2-D Noh, 189                   183 / 186  604 / 372    102 / 133
+//   2-D quadrants, 2427              -       1665 / 1756   938 / 927
+//   3-D blast, 246                 260 / 254  150 / 182    199 / 208
+// One thread per particle takes longer where c-bins are split (`split`: shorter rows).
+// A warp's homes test the union of their windows, 32 particles more per row, and a
+// warp whose homes lie in several rows walks once per row (`runs`).
+struct SearchCosts {
+    double ps[3];   // kSearchDirect, kSearchFilter, kSearchPairs
+};
+inline SearchCosts search_costs(int dim, bool split, double cand, double hits, double passing, double rows, double n_row) {
+    const double tests = cand + 32.0 * rows, runs = 1.0 + 32.0 / (n_row > 1.0 ? n_row : 1.0);
+    SearchCosts c;
+    c.ps[kSearchDirect] = dim == 2 ? 25.0 + 0.85 * cand : split ? 70.0 + 1.3 * cand : 45.0 + 0.85 * cand;
+    c.ps[kSearchFilter] = (130.0 + 0.07 * cand + 6.0 * hits) * runs;
+    c.ps[kSearchPairs] = (dim == 3 ? 38.0 + 0.30 * tests : 24.0 + 0.28 * tests) * runs + 3.0 * (passing < 64.0 ? passing : 64.0);
+    return c;
+}
+// the cheapest of the searches in `allowed` (a bit each)
+inline int cheapest_search(const SearchCosts& c, unsigned allowed) {
+    int best = -1;
+    for (int k = 0; k < 3; ++k)
+        if ((allowed >> k & 1u) && (best < 0 || c.ps[k] < c.ps[best])) best = k;
+    return best;
+}
 
 // precision-independent
 cudaError_t launch_scan(uint32_t* count, uint32_t* start, uint32_t n_keys, uint32_t n_tiles,

@@ -793,7 +793,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) search_kerne
     const uint32_t tag = R<T>::bits(P.w);
     const int inst = tag_inst(b, tag);
     const InstDev& I = b.inst[inst];
-    if (I.tiled || I.filtered) return;   // searched, and its slot_of recorded, by another kernel
+    if (I.tiled || I.search != kSearchDirect) return;   // searched, and its slot_of recorded, by another kernel
     // sorted position by id, read by the move kernel to find a partner
     b.slot_of[I.p_off + (int64_t)tag_id(b, tag)] = (uint32_t)p;
     if (I.staged || absorbed(Q.w)) return;   // searched by the staged kernel, or gone
@@ -3551,6 +3551,7 @@ cudaError_t launch_window_count(const Bufs<T>& b, unsigned long long* total, cud
     template cudaError_t launch_cell_keys<T>(const Bufs<T>&, int32_t*, cudaStream_t);              \
     template cudaError_t launch_moments<T>(const Bufs<T>&, int, cudaStream_t);                     \
     template cudaError_t launch_filtered_search<T>(const Bufs<T>&, cudaStream_t);                  \
+    template cudaError_t launch_pairs_search<T>(const Bufs<T>&, cudaStream_t);                     \
     template cudaError_t launch_cbin_hist<T>(const Bufs<T>&, uint32_t*, unsigned long long*, double*, cudaStream_t); \
     template cudaError_t launch_window_count<T>(const Bufs<T>&, unsigned long long*, cudaStream_t);   \
     template cudaError_t launch_perm<T>(const Bufs<T>&, int32_t*, cudaStream_t);                   \

@@ -123,14 +123,21 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     // The search as kmc_init chooses it (kmc_api.cu, choose_filter), without statistics
     // of the state: mean density, windows of the contact distance and a search cell,
     // each pair once unless many candidates lie within the contact distance.
-    double within = nbar, cand = nbar;
+    double within = nbar, cand = nbar, rows = 1.0, n_rows = 1.0;
     for (int d = 0; d < g.dim; ++d) {
         within *= fmin(2.0 * sqrt(I.R2), fmin(3.0 * g.L[d] / g.n[d], g.L[d]));
         const double k = ceil(sqrt(I.R2) / I.w[d]) + 1.0;   // search cells within the contact distance and a step
         cand *= fmin((2.0 * k + 1.0) * I.w[d], fmin(3.0 * g.L[d] / g.n[d], g.L[d]));
+        if (d + 1 < g.dim) rows *= fmin(2.0 * k + 1.0, fmin(3.0 * I.s[d], I.M[d]));
+        if (d + 1 < g.dim) n_rows *= I.M[d];
     }
     I.sym = sizeof(T) == 4 && within <= 4.0 * kSymPassing ? 1 : 0;
-    I.filtered = sizeof(T) == 8 || filter_pays(cand, I.sym ? 0.25 * fmin(within, cand) : 0.05 * cand) ? 1 : 0;
+    const double near = fmin(within, cand), passing = 0.25 * near;
+    const bool split = I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1;
+    I.search = sizeof(T) == 8 ? kSearchFilter
+                              : cheapest_search(search_costs(g.dim, split, cand, I.sym ? 0.25 * near : 0.1 * cand, passing,
+                                                             rows, (double)n / n_rows), 7u);
+    I.close = passing > kPairsClose ? 1 : 0;
     I.chi = sizeof(T) == 8 ? 1 : 0;
     Bufs<T> b{};
     b.n = n;
@@ -160,8 +167,9 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return KMC_ECUDA;
-    b.filtered = I.filtered;
-    b.any_direct = !I.filtered;
+    b.filtered = I.search == kSearchFilter;
+    b.paired = I.search == kSearchPairs ? (I.close ? 3 : 1) : 0;
+    b.any_direct = I.search == kSearchDirect;
     b.filter_chi = I.chi;
     b.filter_split = filter_split(n, sms);
     b.id_bits = 32;
@@ -180,7 +188,9 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     if (launch_scan(b.count, b.start, n_keys, n_tiles, b.scan_status, b.dyn, b.inst, 1, b.st, g, 0, s) != cudaSuccess)
         return KMC_ECUDA;
     if (launch_scatter<T>(b, s) != cudaSuccess) return KMC_ECUDA;
-    if ((I.filtered ? launch_filtered_search<T>(b, s) : launch_search<T>(b, s)) != cudaSuccess) return KMC_ECUDA;
+    if ((b.filtered ? launch_filtered_search<T>(b, s) : b.paired ? launch_pairs_search<T>(b, s) : launch_search<T>(b, s)) !=
+        cudaSuccess)
+        return KMC_ECUDA;
     best_by_id<T><<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(b, best);
     return cudaGetLastError() == cudaSuccess ? KMC_OK : KMC_ECUDA;
 }

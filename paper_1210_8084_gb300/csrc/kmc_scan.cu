@@ -145,7 +145,11 @@ __device__ void step_bookkeeping(InstDyn* dyn, const InstDev* inst, int n_inst, 
         dyn[i].mom_e[1] = vm > 0.0 ? fixed_exponent(nn * vm * vm) : 120;
         const double wm = nn * 4.0 * sqrt(inst[i].R2) * vm;
         dyn[i].mom_e[2] = wm > 0.0 ? fixed_exponent(wm) : 120;
-        if (inst[i].filtered) filter_constants(dyn[i], inst[i], geo, (float)(vmax * dt), (float)D);
+        dyn[i].p_image = 0;
+        for (int d = 0; d < geo.dim; ++d)
+            if (geo.bc[d] == KMC_BC_PERIODIC && D * 1.001 >= 0.499 * geo.L[d]) dyn[i].p_image = 1;
+        dyn[i].p_slack = (float)(0x1p-19 * D * D);
+        if (inst[i].search == kSearchFilter) filter_constants(dyn[i], inst[i], geo, (float)(vmax * dt), (float)D);
     }
     if (threadIdx.x == 0 && bump) st->step += 1u;
 }
