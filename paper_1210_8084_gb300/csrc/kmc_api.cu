@@ -336,6 +336,21 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
         if (ok) {
             for (int d = 0; d < h->dim; ++d) s[d] = 2;
             I.prune = 1;
+            // The filtered search (no tile parameters asked for) takes fewer rows, each
+            // split finer: its lists cover 8 consecutive particles, so cells of about 5
+            // along the rows keep them compact, and a row costs it a walk of its
+            // own.  Steps at (2, 2, 2) and here, 3-D Sod tubes: 10 particles per c-bin
+            // 1.89 -> 1.35 ms, 20 6.41 -> 5.18, 33 5.45 -> 4.75, 122 11.6 -> 11.1, 200 25.4
+            // -> 22.7; whole c-bins across the rows are slower from 65 on (122: 12.6).
+            // 2-D, (2, 2) and here: 20 per c-bin 1.29 -> 1.15, 125 3.38 -> 3.12, 400 8.03 ->
+            // 7.80.  Small instances keep half c-bins, the grid that callers of
+            // kmc_get_info have seen for them (20 % of a 0.3 ms step at 60,000).
+            if (I.n >= kFineRows && h->cfg.tile_threads == 0 && h->cfg.tile_cap == 0 && h->cfg.tile_split == 0) {
+                const double mean = (double)I.n / (double)h->bins_per_inst;
+                const int across = h->dim == 3 && mean > 64.0 ? 2 : 1;
+                for (int d = 0; d + 1 < h->dim; ++d) s[d] = across;
+                s[h->dim - 1] = std::min(8, std::max(2, (int)lround(mean / (5.0 * across * across))));
+            }
         }
     }
     for (int d = 0; d < 3; ++d) {

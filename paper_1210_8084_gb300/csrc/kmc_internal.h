@@ -24,6 +24,7 @@ constexpr int kTestSlots = 256;        // counters of the pruned tile search's p
 constexpr int kCbinRows = 4;           // rows of search cells per c-bin up to which moments go one warp per c-bin
 constexpr int kPrunedCap = 1888;       // default staging capacity of the pruned tile search (28 B per slot)
                                        // count, Sum v.r_hat
+constexpr int64_t kFineRows = 1 << 18;  // pruned instances from this many particles on: rows of finer cells
 constexpr double kSymPassing = 64.0;   // filtered search: passing candidates per particle up to which a pair is tested once
 constexpr double kPairsClose = 16.0;   // pair search: passing candidates per particle from which pairs are tested
                                        // against the closest so far

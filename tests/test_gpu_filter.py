@@ -104,3 +104,40 @@ def test_filtered_and_per_particle_instances_share_a_handle():
         plain.close()
         off += ns[i]
     batch.close()
+
+
+FINE_ROWS = [
+    # name, n, dim, cells, hi, bc, lam, search cells per c-bin
+    ("few_per_bin", 1 << 18, 3, (40, 16, 16), (1, .4, .4), (WALL, PER, PER), 2e-3, [1, 1, 5]),
+    ("many_per_bin", (1 << 18) + 7, 3, (24, 8, 6), (1, 8 / 24, 6 / 24), (WALL, WALL, PER), 2e-2, [2, 2, 8]),
+    ("plane", 300_001, 2, (60, 60, 1), (1, 1, 1), (PER, WALL, PER), 5e-2, [1, 8, 1]),
+    ("small", (1 << 18) - 1, 3, (40, 16, 16), (1, .4, .4), (WALL, PER, PER), 2e-3, [2, 2, 2]),
+]
+
+
+@pytest.mark.parametrize("case", FINE_ROWS, ids=[c[0] for c in FINE_ROWS])
+def test_rows_of_finer_cells_do_not_change_results(case):
+    """Pruned instances from 2^18 particles on: rows of search cells finer than half
+    c-bins, the candidates and states those of one thread per particle."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import paper_1210_8084_gb300 as k
+    from paper_1210_8084_gb300 import inputs
+    name, n, dim, cells, hi, bc, lam, sub = case
+    lo = (0, 0, 0)
+    pos, vel = inputs.sod_tube(n, seed=5, lo=lo, hi=hi, split=0.5, dim_pos=dim)
+    pos[:, 0] = np.where(pos[:, 0] >= hi[0], lo[0], pos[:, 0])
+    pos, vel = inputs.cast_state(pos, vel, np.float32, lo, hi, bc)
+    out = []
+    for flags in (0, k.KMC_FLAG_NO_TILE_SEARCH):
+        sim = k.Simulation(k.make_config(dim_pos=dim, n_cells=cells, lo=lo, hi=hi, bc=bc, lam=lam, dt=0.2 / cells[0], seed=3,
+                                         precision=32, flags=flags | k.KMC_FLAG_RECORD), pos, vel)
+        if not flags:
+            assert sim.info().tile_prune == 1 and list(sim.info().sub_cells) == sub
+        sim.step(2)
+        out.append((*sim.partners(), *sim.state(), sim.moments()[0]))
+        sim.close()
+    assert (out[0][0] >= 0).mean() > 0.01
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
