@@ -3,7 +3,8 @@
 //
 // Step structure (Sagert et al., Sect. "Simulation setup" and Fig. 2):
 //   search  : closest PoCA candidate per particle over its c-bin neighbourhood
-//             (per particle, or per c-bin block on unsubdivided grids)
+//             (per particle here, or by kmc_filter.cuh / kmc_pairs.cuh; a block per
+//             c-bin where a flag or tile parameters ask for it)
 //   move    : unambiguous pairs, CM scattering, split free flight, walls,
 //             next search key + histogram
 //   scan    : exclusive scan of the key histogram (kmc_scan.cu)
@@ -583,6 +584,11 @@ __device__ __forceinline__ int unwrap(int t, int M, T L, T& shift) {
     return t;
 }
 
+// Per-particle search: threads per block.  A block holds its registers until its
+// longest walk is done: of 32 warps per SM 23 were active with blocks of 256.  16M slab
+// tube, ms: 256 threads 1.13, 128 1.06, 64 1.03, 32 (32 blocks per SM at most) 1.10.
+constexpr int kSearchThreads = 64;
+
 // Every candidate range of one particle.  The last position dimension is the
 // fastest of the key, so a window is a set of rows (x, or x and y) each with
 // one or two contiguous key ranges.  Common case (at most 3 cells per row
@@ -590,7 +596,7 @@ __device__ __forceinline__ int unwrap(int t, int M, T L, T& shift) {
 // loads overlap, then the rows are scanned in turn.  Otherwise rows are
 // visited one at a time.
 // Walk the non-empty row ranges of one particle as one sequence: the ranges
-// sit in shared memory (`rng`, one slot per row, stride kThreads), `mask`
+// sit in shared memory (`rng`, one slot per row, stride kSearchThreads), `mask`
 // marks the non-empty rows, and the next candidate is loaded while the current
 // one is tested.  A lane with short rows goes on to its next row instead of
 // idling until the longest row of its warp is done.  `code` holds the periodic
@@ -609,7 +615,7 @@ __device__ __forceinline__ void walk_rows(const Bufs<T>& b, const GeoT<T>& G, co
     if (mask == 0u) return;
     int r = __ffs(mask) - 1;
     mask &= mask - 1u;
-    int2 rg = rng[r * kThreads];
+    int2 rg = rng[r * kSearchThreads];
     int32_t q = rg.x, qe = rg.y;
     auto row_shift = [&](int row, T& s0, T& s1) {
         const int ix = (DIM == 3) ? row / 3 : row;
@@ -633,7 +639,7 @@ __device__ __forceinline__ void walk_rows(const Bufs<T>& b, const GeoT<T>& G, co
             if (mask != 0u) {
                 r = __ffs(mask) - 1;
                 mask &= mask - 1u;
-                rg = rng[r * kThreads];
+                rg = rng[r * kSearchThreads];
                 q = rg.x;
                 qe = rg.y;
                 row_shift(r, s0, s1);
@@ -722,7 +728,7 @@ __device__ __forceinline__ void scan_window(const Bufs<T>& b, const GeoT<T>& G, 
             for (int r = 0; r < NR; ++r) {
                 if (SYM) q0[r] = max(q0[r], self + 1);
                 if (q1[r] > q0[r]) {
-                    rng[r * kThreads] = make_int2(q0[r], q1[r]);
+                    rng[r * kSearchThreads] = make_int2(q0[r], q1[r]);
                     mask |= 1u << r;
                 }
             }
@@ -781,11 +787,11 @@ __device__ __forceinline__ void scan_window(const Bufs<T>& b, const GeoT<T>& G, 
 // tests every candidate of a full window and stores its key.  Every particle
 // records its sorted position by id (slot_of) for the move kernel.
 template <typename T, int DIM>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) search_kernel(Bufs<T> b) {
+__global__ void __launch_bounds__(kSearchThreads, (sizeof(T) == 4 ? 4 : 2) * kThreads / kSearchThreads) search_kernel(Bufs<T> b) {
     using V = typename Vec4<T>::type;
     constexpr bool kSym = sizeof(T) == 4;
     const GeoT<T>& G = b.g;   // kernel parameter: constant bank
-    __shared__ int2 rng[(DIM == 3 ? 9 : 3) * kThreads];
+    __shared__ int2 rng[(DIM == 3 ? 9 : 3) * kSearchThreads];
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= b.n) return;
     const V P = b.posA[p];
@@ -834,7 +840,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) search_kerne
                 const int32_t q1 = (int32_t)min(b.start[rows[r] + 3u], nmax);
                 if (r == 0) q0 = max(q0, (int32_t)p + 1);
                 if (q1 > q0) {
-                    rng_t[r * kThreads] = make_int2(q0, q1);
+                    rng_t[r * kSearchThreads] = make_int2(q0, q1);
                     mask |= 1u << r;
                 }
             }
@@ -3112,7 +3118,7 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(Bufs<T> b, int use_vi
 // its sums, with no atomics (fixed-point sums do not depend on their order).  A
 // warp per c-bin left most lanes without a particle where c-bins hold a few (the
 // reduction costs the same): 8 lanes below 24 particles on average, 16 below 96.
-// 8M particles at 8 per c-bin, GB300: 0.662 -> 0.262 ms; 21M at 20 0.846 -> 0.404 ms.
+// 8M particles at 8 per c-bin, GB300: 0.662 -> 0.204 ms; 21M at 20 0.846 -> 0.363 ms.
 template <typename T, int DIM, bool RADIAL, int LANES>
 __global__ void __launch_bounds__(kThreads) moments_cbin_kernel(Bufs<T> b, int use_virial) {
     using V = typename Vec4<T>::type;
@@ -3363,7 +3369,11 @@ cudaError_t launch_search(const Bufs<T>& b, cudaStream_t s) {
     }
     // besides the direct search it records slot_of for the particles of every
     // instance that is not tiled (staged ones included)
-    if (b.any_direct || b.n_stage_tiles > 0) KMC_DIM_DISPATCH(b.geo.dim, search_kernel, b);
+    if (b.any_direct || b.n_stage_tiles > 0) {
+        const unsigned blocks = (unsigned)((b.n + kSearchThreads - 1) / kSearchThreads);
+        if (b.geo.dim == 3) search_kernel<T, 3><<<blocks, kSearchThreads, 0, s>>>(b);
+        else search_kernel<T, 2><<<blocks, kSearchThreads, 0, s>>>(b);
+    }
     return cudaGetLastError();
 }
 
