@@ -369,8 +369,8 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
 // The binary32 filter looks at each pair once, its threshold then staying R^2, or,
 // where many candidates pass, at every home's whole window with a threshold that
 // falls to its closest candidate: twice the pairs, but few of them left (a tenth
-// at 150-270 particles per c-bin of the quadrant workload).  Binary64 always filters (its exact test runs at 1/64
-// of the binary32 rate), by criterion 1 too.
+// at 150-270 particles per c-bin of the quadrant workload).  Binary64 (its exact test runs at 1/64 of the
+// binary32 rate) filters by criterion 1 too, unless a window holds few candidates.
 SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms, double occ) {
     const double dt0 = (I.adaptive && vmax > 0.0) ? I.dx_min / vmax : I.dt;
     const double R = sqrt(I.R2), reach = 1.001 * (R + 2.0 * vmax * dt0), rho = sqrt(I.R2 + 1.2 * vrms * vrms * dt0 * dt0);
@@ -390,7 +390,6 @@ SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms,
         h->filter_chi = 1;   // criterion 1 leaves about the passing ones
         hits = std::min(hits, 4.0 * passing);
     }
-    if (h->precision == 64) h->filter_chi = 1;
     double rows = 1.0, n_row = occ * h->geo.n[h->dim - 1];
     for (int d = 0; d + 1 < h->dim; ++d) {
         const double k = ceil((reach + 1e-5 * h->geo.L[d]) / I.w[d]);
@@ -398,11 +397,17 @@ SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms,
         n_row /= I.s[d];
     }
     I.close = passing > kPairsClose ? 1 : 0;
-    return search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, cand, hits, passing, rows, n_row);
+    if (h->precision == 64) {
+        h->filter_chi = 1;
+        return search_costs64((double)h->n, cand, n_row);
+    }
+    bool wraps = false;   // with room for v_max to grow (InstDyn::p_image)
+    for (int d = 0; d < h->dim; ++d) wraps = wraps || (h->geo.bc[d] == KMC_BC_PERIODIC && reach > 0.4 * h->geo.L[d]);
+    return search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, wraps, (double)h->n, cand, hits, passing, rows, n_row);
 }
 
-// The searches of a handle's instances: pruned ones and binary64 are filtered, the
-// others by the set of searches that costs least.  A further search reads every
+// The searches of a handle's instances: pruned ones are filtered, the others take the
+// set of searches that costs least.  A further search reads every
 // particle once more (6 ps each: a 158M-particle ensemble took 30.0 ms with the three
 // cheapest per instance and 27.9 ms with one).  A handle with pruned instances uses
 // no pair search.
@@ -415,8 +420,8 @@ void choose_searches(kmc_handle* h, const std::vector<SearchCosts>& cost) {
     }
     unsigned best = 1u << kSearchFilter;
     double least = INFINITY;
-    for (unsigned set = 1; set < 8 && h->precision == 32; ++set) {
-        if (prune && (set & (1u << kSearchPairs))) continue;
+    for (unsigned set = 1; set < 8; ++set) {
+        if ((prune || h->precision == 64) && (set & (1u << kSearchPairs))) continue;
         double sum = 0.0;
         unsigned used = prune ? 1u << kSearchFilter : 0u;
         for (int i = 0; i < h->n_inst; ++i) {

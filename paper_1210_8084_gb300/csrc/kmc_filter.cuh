@@ -30,11 +30,12 @@
 // below 2^-17 D^2 with D the reach R + 2 v_max dt) and by that of the product's
 // sum (16 terms of 12 X^2 in all: 2^-18 of it).  kmc_scan.cu holds the constants.
 //
-// Bound by instruction issue and latency.  Tile searches before -> this search,
-// GB300, ms per step: 3-D Sod tube, 512M particles 423 -> 253, 16M 14.6 -> 8.4, 21M
-// at 20 per c-bin 25.0 -> 6.3; Sedov blast, 8M 15.3 -> 1.4; quadrants, 64M 182 -> 117;
-// binary64 slab tube, 200k 2.33 -> 0.30.  Per 32 homes of the 16M tube: 431 tiles of 8
-// candidates in the window, 135 past the box check, 411 pairs past the filter.
+// Bound by instruction issue (71 % of the slots, 10,400 instructions per 32 homes of the
+// 16M tube).  The searches it replaced -> this one, GB300, ms per step: 3-D Sod tube,
+// 512M particles 423 -> 191, 16M 14.6 -> 6.3, 21M at 20 per c-bin 25.0 -> 3.6; Sedov
+// blast, 8M 15.3 -> 1.14; binary64 slab tube, 200k 2.33 -> 0.27.  Per 32 homes of the 16M
+// tube: 431 tiles of 8 candidates in the window, 135 past the box check, 411 pairs
+// past the filter.
 #pragma once
 
 #include "kmc_kernels.cuh"
@@ -344,7 +345,7 @@ struct FiltWarp {
 //   both keys (each pair once), threshold R^2.  Otherwise the whole window, the
 //   outcome kept by the home alone and the threshold lowered to its closest
 //   candidate: better where many candidates of the window pass (a contact
-//   distance about as wide as the c-bins); binary64 always.
+//   distance about as wide as the c-bins); binary64.
 //   CHI: two more products give the signs of a = r0.s and f = r1.s (s = v_rel
 //   dt), criterion 1 itself: worth it where the contact distance is wider than a
 //   step's displacement, so that F < R^2 keeps most of the near pairs.
@@ -886,7 +887,7 @@ cudaError_t launch_filtered(const Bufs<T>& b, cudaStream_t s) {
 template <typename T>
 cudaError_t launch_filtered_search(const Bufs<T>& b, cudaStream_t s) {
     if (b.n == 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4)   // binary64 always filters by criterion 1
+    if constexpr (sizeof(T) == 4)   // binary64 filters by criterion 1 too
         if (!b.filter_chi) return b.geo.dim == 3 ? launch_filtered<T, 3, false>(b, s) : launch_filtered<T, 2, false>(b, s);
     return b.geo.dim == 3 ? launch_filtered<T, 3, true>(b, s) : launch_filtered<T, 2, true>(b, s);
 }

@@ -63,7 +63,7 @@ struct InstDev {
     // shared memory before the search
     int staged;
     int tiled;           // search cells are the c-bins: one block per cell (tile_search_kernel)
-    int prune;           // tiled, binary32: candidate clusters out of a warp's reach are skipped
+    int prune;           // binary32: searched on cells finer than the c-bins, candidates out of reach skipped
     int search;          // kSearch...: its search, unless tiled or staged
     int chi;             // filtered search: criterion 1 filters too (the same for every instance of a handle)
     int sym;             // filtered search, binary32: each pair tested once, by its lower position
@@ -280,7 +280,7 @@ inline int rank_launches(int64_t n, uint32_t n_keys) {
     return mean >= kRankMeanLarge ? 2 : mean >= kRankMean ? 1 : 0;
 }
 
-// Estimated costs of the three searches of a binary32 instance in ps per particle,
+// Estimated costs of the three searches of a binary32 instance in ps per particle (binary64 below),
 // fitted on a GB300 to 36 states (slab tubes of 0.3M-16M particles with R from one to
 // sixty c-bins, 2-D implosions and quadrants, 3-D blasts).  `cand`: candidates in
 // a particle's window; `hits`: those that pass the filter; `passing`: those that meet;
@@ -293,17 +293,41 @@ inline int rank_launches(int64_t n, uint32_t n_keys) {
 //   2-D quadrants, 2427              -       1665 / 1756   938 / 927
 //   3-D blast, 246                 260 / 254  150 / 182    199 / 208
 // One thread per particle takes longer where c-bins are split (`split`: shorter rows).
+// To these come the times of a single walk, which small handles (`n_all` particles)
+// take whole; us measured / estimated for tubes of 10,000-110,000 particles: 10 candidates
+// 23 / 23, 93-170 / 85-120, 46-54 / 36-40; 223 candidates 115 / 119, 69 / 76, 51 / 69. A
+// window that may reach around a periodic box (`wraps`) makes the pair search decide
+// every pair exactly (4,900 particles, 440 candidates: 138 us, 113, 1240).
 // A warp's homes test the union of their windows, 32 particles more per row, and a
 // warp whose homes lie in several rows walks once per row (`runs`).
 struct SearchCosts {
     double ps[3];   // kSearchDirect, kSearchFilter, kSearchPairs
 };
-inline SearchCosts search_costs(int dim, bool split, double cand, double hits, double passing, double rows, double n_row) {
+inline SearchCosts search_costs(int dim, bool split, bool wraps, double n_all, double cand, double hits, double passing,
+                                double rows, double n_row) {
     const double tests = cand + 32.0 * rows, runs = 1.0 + 32.0 / (n_row > 1.0 ? n_row : 1.0);
     SearchCosts c;
     c.ps[kSearchDirect] = dim == 2 ? 25.0 + 0.85 * cand : split ? 70.0 + 1.3 * cand : 45.0 + 0.85 * cand;
     c.ps[kSearchFilter] = (130.0 + 0.07 * cand + 6.0 * hits) * runs;
     c.ps[kSearchPairs] = (dim == 3 ? 38.0 + 0.30 * tests : 24.0 + 0.28 * tests) * runs + 3.0 * (passing < 64.0 ? passing : 64.0);
+    c.ps[kSearchDirect] += (20.0 + 0.27 * cand) * 1e6 / n_all;
+    c.ps[kSearchFilter] += (45.0 + 10.0 * runs + 0.3 * hits) * 1e6 / n_all;
+    c.ps[kSearchPairs] += (35.0 + 0.04 * cand) * 1e6 / n_all;
+    if (wraps) c.ps[kSearchPairs] *= 20.0;
+    return c;
+}
+// Binary64: one thread per particle or filtered, per particle of a handle of n_all.  Up to
+// some 80,000 particles a search is one wave, its time that of a particle's walk or of a
+// group's runs.  us per search, measured / estimated, one thread per particle and filtered
+// (slab tubes): 30,000 particles, 10 candidates, 13 per row of cells 89 / 122, 236 / 284;
+// 11,000, 112, 21 per row 380 / 505, 328 / 198; 97,000, 43, 21 per row 554 / 490, 247 / 267;
+// 1M, 11, 33 per row 1190 / 1270, 940 / 950; 1M, 67, 65 per row 4600 / 4800, 1000 / 910.
+inline SearchCosts search_costs64(double n_all, double cand, double n_row) {
+    const double runs = 1.0 + 32.0 / (n_row > 1.0 ? n_row : 1.0);
+    SearchCosts c;
+    c.ps[kSearchDirect] = (45.0 + 3.4 * cand) * 1e6 / n_all + 500.0 + 60.0 * cand;
+    c.ps[kSearchFilter] = 75.0 * runs * 1e6 / n_all + 800.0;
+    c.ps[kSearchPairs] = c.ps[kSearchDirect] + c.ps[kSearchFilter];   // binary32 only
     return c;
 }
 // the cheapest of the searches in `allowed` (a bit each)

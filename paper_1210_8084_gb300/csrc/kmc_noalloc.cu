@@ -120,23 +120,28 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
         return q;
     };
     const size_t nv = ((size_t)(n > 0 ? n : 1) + 31) / 32 * 32;   // whole tiles of the filtered search
-    // The search as kmc_init chooses it (kmc_api.cu, choose_filter), without statistics
+    // The search as kmc_init chooses it (kmc_api.cu, estimate_search), without statistics
     // of the state: mean density, windows of the contact distance and a search cell,
     // each pair once unless many candidates lie within the contact distance.
     double within = nbar, cand = nbar, rows = 1.0, n_rows = 1.0;
+    bool wraps = false;
     for (int d = 0; d < g.dim; ++d) {
         within *= fmin(2.0 * sqrt(I.R2), fmin(3.0 * g.L[d] / g.n[d], g.L[d]));
         const double k = ceil(sqrt(I.R2) / I.w[d]) + 1.0;   // search cells within the contact distance and a step
         cand *= fmin((2.0 * k + 1.0) * I.w[d], fmin(3.0 * g.L[d] / g.n[d], g.L[d]));
         if (d + 1 < g.dim) rows *= fmin(2.0 * k + 1.0, fmin(3.0 * I.s[d], I.M[d]));
         if (d + 1 < g.dim) n_rows *= I.M[d];
+        wraps = wraps || (g.bc[d] == KMC_BC_PERIODIC && k * I.w[d] > 0.4 * g.L[d]);
     }
     I.sym = sizeof(T) == 4 && within <= 4.0 * kSymPassing ? 1 : 0;
     const double near = fmin(within, cand), passing = 0.25 * near;
     const bool split = I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1;
-    I.search = sizeof(T) == 8 ? kSearchFilter
-                              : cheapest_search(search_costs(g.dim, split, cand, I.sym ? 0.25 * near : 0.1 * cand, passing,
-                                                             rows, (double)n / n_rows), 7u);
+    const double n_row = (double)n / n_rows;
+    I.search = n == 0 ? kSearchDirect
+               : sizeof(T) == 8
+                   ? cheapest_search(search_costs64((double)n, cand, n_row), 1u << kSearchDirect | 1u << kSearchFilter)
+                   : cheapest_search(search_costs(g.dim, split, wraps, (double)n, cand, I.sym ? 0.25 * near : 0.1 * cand, passing,
+                                                    rows, n_row), 7u);
     I.close = passing > kPairsClose ? 1 : 0;
     I.chi = sizeof(T) == 8 ? 1 : 0;
     Bufs<T> b{};
