@@ -67,8 +67,11 @@ extern "C" {
 #define KMC_FLAG_RECORD 1   /* keep each particle's closest candidate and partner of the last step */
 #define KMC_FLAG_NO_GRAPH 2 /* launch kernels directly instead of replaying a captured CUDA graph (by default
                              * kmc_step launches one graph that loops over all its steps on the device) */
+/* The search of an instance (one particle per thread, filtered by tensor-core products, or a lane per particle
+ * against staged pairs) is chosen by its estimated cost.  The next two flags, KMC_FLAG_NO_TILE_PRUNE and the tile
+ * parameters of kmc_config ask for one of the other searches instead; speed only, never results. */
 #define KMC_FLAG_STAGED_SEARCH 4 /* stage tile neighbourhoods in shared memory (3-D; same results as the direct search) */
-#define KMC_FLAG_NO_TILE_SEARCH 8 /* search unsubdivided grids per particle too (default: one block per c-bin; same results) */
+#define KMC_FLAG_NO_TILE_SEARCH 8 /* one particle per thread for every instance (same results) */
 #define KMC_FLAG_VELOCITY_2D 32  /* dim_pos = 2 only: velocities in the (x, y) plane (the paper's 2-D runs, f = 2,
                                   * gamma = 2): v_z must be 0, outgoing directions isotropic in the plane
                                   * (azimuth 2 pi u2 of the pair's draw), T = m v_rms^2 / 2 */
@@ -82,14 +85,13 @@ extern "C" {
                             * must be 0 or 1).  Collided particles count as paired in the moments (zero virial);
                             * kmc_get_partners reports -1 */
 #define KMC_FLAG_RADIAL_MOMENT 128 /* also accumulate the radial velocity per c-bin (KMC_MOM_RADIAL, Eq. vel_r) */
-#define KMC_FLAG_NO_TILE_PRUNE 256 /* binary32: no pruned tile search.  By default an instance whose automatic
-                                    * search cells would be its c-bins (the reach exceeds half a c-bin), whose contact
-                                    * distance R is at most half the narrowest c-bin and whose periodic dimensions
-                                    * have 6 c-bins or more searches on half c-bins (sub_cells 2 per position
-                                    * dimension) with one block per c-bin, where each group of 32 homes skips every
-                                    * cluster of 4 candidates whose swept box (positions over the step) stays farther
-                                    * than R, plus a rounding margin, from the group's, and each home then every
-                                    * remaining cluster that stays as far from its own; same results */
+#define KMC_FLAG_NO_TILE_PRUNE 256 /* binary32: search cells that are the c-bins, one block per c-bin, where by default
+                                    * candidates out of reach are skipped on finer cells: in an instance whose
+                                    * automatic search cells would be its c-bins (the reach exceeds half a c-bin),
+                                    * whose contact distance R is at most half the narrowest c-bin and whose periodic
+                                    * dimensions have 6 c-bins or more.  Those are half c-bins (sub_cells 2 per
+                                    * position dimension), or from 2^18 particles on whole or half c-bins across and
+                                    * 2 to 8 cells along the last position dimension; same results */
 #define KMC_FLAG_ADAPTIVE_DT 16  /* timestep dt(t) = dx_min / v_max(t) of each step's start state (Sect. "Simulation
                                   * setup"; dx_min the smallest c-bin width, v_max the largest speed of the instance,
                                   * |v|^2 = fma(vz, vz, fma(vy, vy, vx vx)) in the state precision, the quotient in
@@ -135,8 +137,9 @@ typedef struct kmc_config {
     double occupancy_target; /* automatic subdivision: particles per search cell aimed at (0 = 0.5) */
     int flags;          /* KMC_FLAG_* */
     double radial_center[3]; /* centre of the radial velocity moment (KMC_MOM_RADIAL), finite */
-    int tile_threads;   /* search of unsubdivided grids (one block per c-bin): threads per block, a
-                         * multiple of 32 from 64 to 256 (0 = 256); speed only, never results */
+    int tile_threads;   /* the three: not 0 asks for one block per c-bin where search cells are the c-bins
+                         * (or, pruned, their halves).  Threads per block, a multiple of 32 from 64 to
+                         * 256 (0 = 256); speed only, never results */
     int tile_cap;       /* the same: candidates staged in shared memory at once, even, 64 ... 6144 in
                          * binary32, 64 ... 3072 in binary64 (0 = 1536 / 768, 48 KiB); speed only */
     int tile_split;     /* the same, binary32: blocks that share one c-bin's candidates, 1 ... 8 (0 = 1);
@@ -148,12 +151,11 @@ typedef struct kmc_config {
  * restricted to the search cells that can hold a candidate).  Synchronises. */
 KMC_API int kmc_window_size(kmc_handle* h, double* mean_candidates);
 
-/* Pair tests the binary32 tile search has evaluated since kmc_init with its
- * pruning (KMC_FLAG_NO_TILE_PRUNE unset): 4 for every (home, cluster of 4
- * staged candidates) pair whose boxes meet (padding slots of a window row's
- * last cluster included).  0 for handles without that search.
- * The plain tile search tests (C_p - 1) / 2 pairs per particle, C_p from
- * kmc_window_size.  Synchronises the handle's stream. */
+/* Pair tests evaluated since kmc_init in instances that skip candidates out of
+ * reach (kmc_info.tile_prune): the pairs left by the filter, each tested exactly;
+ * with tile parameters, 4 for every (home, cluster of 4 staged candidates) pair
+ * whose boxes meet.  0 for other handles, whose window holds (C_p - 1) / 2 pairs
+ * per particle, C_p from kmc_window_size.  Synchronises the handle's stream. */
 KMC_API int kmc_tile_tests(kmc_handle* h, double* tests);
 
 /* Read-only description of a handle (kmc_get_info). */
@@ -184,8 +186,8 @@ typedef struct kmc_info {
     int graph_mode;          /* how the last kmc_step ran: 2 = one CUDA graph for all its steps (a device-side
                               * loop counter drives a conditional while node), 1 = one graph per step,
                               * 0 = kernel by kernel (KMC_FLAG_NO_GRAPH, or before the first kmc_step) */
-    int tile_prune;          /* 1: the binary32 tile search skips candidate clusters out of reach (for some
-                              * instance) */
+    int tile_prune;          /* 1: some binary32 instance skips candidates out of reach on cells finer than its
+                              * c-bins (KMC_FLAG_NO_TILE_PRUNE) */
 } kmc_info;
 
 /* Create a simulation.  pos and vel are n x 3 row-major arrays of float
@@ -206,8 +208,8 @@ KMC_API int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const vo
 KMC_API int kmc_step(kmc_handle* h, int nsteps, int want_moments);
 
 /* Phases of one step, in launch order, for kmc_step_profiled. */
-#define KMC_PHASE_SEARCH 0   /* closest candidate per particle (criteria 1-3), one thread per particle */
-#define KMC_PHASE_TILE 1     /* the same, one block per c-bin, for grids whose search cells are the c-bins */
+#define KMC_PHASE_SEARCH 0   /* closest candidate per particle (criteria 1-3) */
+#define KMC_PHASE_TILE 1     /* the same, one block per c-bin, where a flag or tile parameters ask for it */
 #define KMC_PHASE_MOVE 2     /* pairs, scattering, free flight, walls, next key and histogram */
 #define KMC_PHASE_SCAN 3     /* exclusive scan of the key histogram */
 #define KMC_PHASE_SCATTER 4  /* counting-sort scatter into (key, id) order */
@@ -276,10 +278,10 @@ KMC_API int kmc_get_partners(kmc_handle* h, int32_t* best, int32_t* partner, int
 /* Pick the implementation parameters of the search for a configuration by
  * measurement (the paper has no counterpart: these parameters change speed
  * only, never results).  For each candidate setting -- automatic subdivision
- * at several occupancy targets, the per-c-bin tile search (with several
- * threads per c-bin block and staging capacities) or the per-particle search
- * where the grid is not subdivided, and the shared-memory staged search for
- * 3-D grids -- a handle is created from (cfg, n, pos, vel, where) as in
+ * at several occupancy targets with the search chosen by cost, the per-c-bin
+ * tile search (with several threads per c-bin block and staging capacities) or the
+ * per-particle search where the grid is not subdivided, and the shared-memory
+ * staged search for 3-D grids -- a handle is created from (cfg, n, pos, vel, where) as in
  * kmc_init, warmed up for one step and timed over trial_steps >= 1 steps with
  * CUDA events on its stream, then freed; the caller's data are only read.
  * *best receives a copy of *cfg with occupancy_target, tile_threads, tile_cap,
