@@ -744,7 +744,7 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
     };
 
     // particle buffers
-    const size_t nv = (size_t)std::max<int64_t>(n, 1);
+    const size_t nv = buffer_rows(n);
     if ((rc = dev_alloc(h, &h->posA, nv * vec_size(h)))) return bail(rc);
     if ((rc = dev_alloc(h, &h->velA, nv * vec_size(h)))) return bail(rc);
     if ((rc = dev_alloc(h, &h->posB, nv * vec_size(h)))) return bail(rc);

@@ -259,6 +259,10 @@ cudaError_t launch_dsmc(const Bufs<T>& b, cudaStream_t s);     // random-partner
 template <typename T>
 cudaError_t launch_cbin_hist(const Bufs<T>& b, uint32_t* hist, unsigned long long* vmax2, double* sample, cudaStream_t s);
 
+// Particles the buffers of a state of n hold: whole groups of 32, so that the filtered
+// search's operands of a last tile of 8, and that tile's box, lie inside them.
+inline size_t buffer_rows(int64_t n) { return ((size_t)(n > 0 ? n : 1) + 31) / 32 * 32; }
+
 // log2 of the warps that share a group of 32 homes of the filtered search: a
 // small system has too few groups to fill the chip, so up to eight warps (a
 // block) take one group, until about 16 warps per SM are busy.

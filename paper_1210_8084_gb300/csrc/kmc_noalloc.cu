@@ -119,7 +119,7 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
         off += align256(bytes);
         return q;
     };
-    const size_t nv = ((size_t)(n > 0 ? n : 1) + 31) / 32 * 32;   // whole tiles of the filtered search
+    const size_t nv = buffer_rows(n);
     // The search as kmc_init chooses it (kmc_api.cu, estimate_search), without statistics
     // of the state: mean density, windows of the contact distance and a search cell,
     // each pair once unless many candidates lie within the contact distance.
