@@ -306,6 +306,20 @@ KMC_API int kmc_autotune(const kmc_config* cfg, int64_t n, const void* pos, cons
  * the hold, the cap and the error.  tile = -1 only sets the cap.  Synchronises. */
 KMC_API int kmc_test_hold_scan(kmc_handle* h, int tile, uint32_t spin_cap);
 
+/* The search of one instance, as kmc_init chose it (speed only, never results): *search is one of KMC_SEARCH_*,
+ * *form (may be NULL) its KMC_FORM_* bits.  KMC_SEARCH_PARTICLE for instances without particles and for
+ * KMC_FLAG_DSMC, which searches nothing.  Reads host memory only.  KMC_EINVAL for an instance that is none. */
+#define KMC_SEARCH_PARTICLE 0    /* one particle per thread */
+#define KMC_SEARCH_FILTER 1      /* tensor-core filter, then exact tests */
+#define KMC_SEARCH_PAIRS 2       /* a lane per particle against staged pairs of candidates */
+#define KMC_SEARCH_TILE 3        /* one block per c-bin */
+#define KMC_SEARCH_TILE_PRUNED 4 /* the same on half c-bins, candidates out of reach skipped */
+#define KMC_SEARCH_STAGED 5      /* tile neighbourhoods in shared memory */
+#define KMC_FORM_CLOSE 1         /* pairs: also tested against the closest candidates so far */
+#define KMC_FORM_CRITERION1 2    /* filter: by the sign of the approach too */
+#define KMC_FORM_ONCE 4          /* filter: each pair once, by its lower position */
+KMC_API int kmc_get_search(kmc_handle* h, int instance, int* search, int* form);
+
 /* Closest-candidate search without any allocation.  The paper has no
  * counterpart: this entry point exists for callers that may not allocate
  * device memory themselves or through this library, e.g. a host framework

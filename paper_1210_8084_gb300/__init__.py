@@ -44,6 +44,15 @@ KMC_MOM_RAW = 1
 KMC_MOM_DERIVED = 2
 KMC_MOM_GLOBAL = 4
 KMC_MOM_RADIAL = 8
+KMC_SEARCH_PARTICLE = 0
+KMC_SEARCH_FILTER = 1
+KMC_SEARCH_PAIRS = 2
+KMC_SEARCH_TILE = 3
+KMC_SEARCH_TILE_PRUNED = 4
+KMC_SEARCH_STAGED = 5
+KMC_FORM_CLOSE = 1
+KMC_FORM_CRITERION1 = 2
+KMC_FORM_ONCE = 4
 KMC_NPHASES = 7
 PHASES = ("search", "tile", "move", "scan", "scatter", "moments", "finalize")
 
@@ -51,7 +60,7 @@ ABI_FUNCTIONS = (
     "kmc_init", "kmc_step", "kmc_moments", "kmc_moments_size", "kmc_free", "kmc_sync",
     "kmc_last_error", "kmc_get_info", "kmc_get_state", "kmc_set_state", "kmc_get_cell_keys",
     "kmc_get_partners", "kmc_step_profiled", "kmc_find_partners_noalloc", "kmc_window_size", "kmc_autotune",
-    "kmc_get_perm", "kmc_test_hold_scan", "kmc_tile_tests",
+    "kmc_get_perm", "kmc_test_hold_scan", "kmc_tile_tests", "kmc_get_search",
 )
 KMC_STATIC_MAX_PARTICLES = 262144
 
@@ -169,6 +178,8 @@ def _load():
     L.kmc_window_size.restype = ctypes.c_int
     L.kmc_tile_tests.argtypes = [H, ctypes.POINTER(ctypes.c_double)]
     L.kmc_tile_tests.restype = ctypes.c_int
+    L.kmc_get_search.argtypes = [H, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]
+    L.kmc_get_search.restype = ctypes.c_int
     L.kmc_find_partners_noalloc.argtypes = [ctypes.POINTER(KmcConfig), ctypes.c_int64, vp, vp, vp]
     L.kmc_find_partners_noalloc.restype = ctypes.c_int
     L.kmc_autotune.argtypes = [ctypes.POINTER(KmcConfig), ctypes.c_int64, vp, vp, ctypes.c_int, ctypes.c_int,
@@ -301,6 +312,13 @@ def kmc_tile_tests(h):
     return v.value
 
 
+def kmc_get_search(h, instance=0):
+    """(KMC_SEARCH_*, KMC_FORM_* bits) of an instance."""
+    search, form = ctypes.c_int(), ctypes.c_int()
+    _check(load().kmc_get_search(h, int(instance), ctypes.byref(search), ctypes.byref(form)), h)
+    return search.value, form.value
+
+
 def kmc_find_partners_noalloc(cfg, n, pos, vel, best):
     """Closest candidate of every particle of a device-resident state, with no
     allocation (scratch in the library's fixed device array).  pos, vel, best
@@ -416,6 +434,9 @@ class Simulation:
 
     def tile_tests(self):
         return kmc_tile_tests(self.h)
+
+    def search(self, instance=0):
+        return kmc_get_search(self.h, instance)
 
     def state(self):
         pos = np.zeros((self.n, 3), dtype=self.dtype)

@@ -1207,6 +1207,22 @@ int kmc_get_info(kmc_handle* h, kmc_info* info) {
     return KMC_OK;
 }
 
+int kmc_get_search(kmc_handle* h, int instance, int* search, int* form) {
+    if (!h || !search) return fail(h, KMC_EINVAL, "NULL argument");
+    if (instance < 0 || instance >= h->n_inst) return fail(h, KMC_EINVAL, "no such instance");
+    static_assert(kSearchDirect == KMC_SEARCH_PARTICLE && kSearchFilter == KMC_SEARCH_FILTER &&
+                      kSearchPairs == KMC_SEARCH_PAIRS,
+                  "search numbers");
+    const InstDev& I = h->inst_h[(size_t)instance];
+    *search = I.staged ? KMC_SEARCH_STAGED : I.tiled ? (I.prune ? KMC_SEARCH_TILE_PRUNED : KMC_SEARCH_TILE) : I.search;
+    if (form) {
+        *form = 0;
+        if (*search == KMC_SEARCH_PAIRS && (h->paired & 2)) *form = KMC_FORM_CLOSE;   // one form for the handle
+        if (*search == KMC_SEARCH_FILTER) *form = (I.chi ? KMC_FORM_CRITERION1 : 0) | (I.sym ? KMC_FORM_ONCE : 0);
+    }
+    return KMC_OK;
+}
+
 int kmc_window_size(kmc_handle* h, double* mean_candidates) {
     if (!h || !mean_candidates) return fail(h, KMC_EINVAL, "NULL argument");
     *mean_candidates = 0.0;
