@@ -194,7 +194,10 @@ __global__ void __launch_bounds__(32, kPairsBlocks) pairs_search_kernel(Bufs<flo
                                     const unsigned long long ki = partner_key<float>(d2, W.tag[e]),
                                                              kj = partner_key<float>(d2, __float_as_uint(Pi.w));
                                     if (ki < W.key[i]) atomicMin(&W.key[i], ki);
-                                    if (!CLOSE || -d2 >= W.least[e]) atomicMin(&b.bkey[base + e], kj);
+                                    // farther than its closest so far: not offered.  A bound of R^2 rules
+                                    // nothing out: the rounded d^2 of a pair that meets may lie above it
+                                    if (!CLOSE || W.least[e] <= -R2 || -d2 >= W.least[e])
+                                        atomicMin(&b.bkey[base + e], kj);
                                 }
                             }
                         }
