@@ -866,6 +866,7 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         for (auto& I : h->inst_h) {
             if (dsmc) {   // no closest-approach search at all
                 I.staged = I.tiled = 0;
+                I.search = kSearchDirect;
                 continue;
             }
             if (choose) {
