@@ -50,7 +50,8 @@ constexpr int kFiltChunks = 32;   // chunks whose words may be queued or in test
 constexpr uint32_t kTilePart = 0x80000000u;   // listed tile that reaches past its row's range
 constexpr uint32_t kTileOwn = 0x40000000u;    // listed tile that holds some of the homes (symmetric search)
 constexpr uint32_t kTileMask = 0x0fffffffu;   // its number (below 2^28: fewer than 2^31 particles)
-constexpr float kNoHit = 60000.f;             // own term of a row that has no pair: no sum falls below zero
+constexpr float kNoHit = 60000.f;             // own term of a row that has no pair: no sum falls below zero; with the
+                                              // sign flipped, of one whose margin lets every pair pass
 
 __device__ __forceinline__ uint32_t pack_half2(float a, float b) { return half2_bits(__floats2half2_rn(a, b)); }
 __device__ __forceinline__ float2 unpack_half2(uint32_t u) {
@@ -193,9 +194,9 @@ __global__ void __launch_bounds__(kThreads) filter_prep_kernel(Bufs<T> b) {
         if constexpr (CHI) {
             const ChiTerms t = chi_terms(X, S);
             const float c = fmaf(D.f_c1, sl, D.f_c0);
-            const uint32_t nf = split_half2(t.ys + c);
+            const uint32_t nf = split_half2(fminf(t.ys + c, kNoHit));
             op = make_uint4(t.xy[0], t.xy[1], t.xy[2], split_half2(t.xy_ - share));
-            op2 = make_uint4(lo_lo(t.s[0], nf), lo_lo(t.s[1], nf >> 16), t.s[2], split_half2(t.xs - c));
+            op2 = make_uint4(lo_lo(t.s[0], nf), lo_lo(t.s[1], nf >> 16), t.s[2], split_half2(fmaxf(t.xs - c, -kNoHit)));
         } else {
             const PathTerms t = path_terms(X, S);
             const uint32_t m01 = t.mh01 ^ kNegHalves, m2 = t.mh2 ^ kNegHalves;
@@ -426,7 +427,8 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
                     thr = fminf(thr, fmaf(d2 * (1.f + 0x1p-20f), D.f_sc2, fmaf(D.f_rt, sqrtf(d2), D.f_slack)));
                 }
             }
-            const uint32_t w = split_half2(fminf(nI - thr, kNoHit));
+            // (a contact distance beyond the frames' width: within binary16's range all the same)
+            const uint32_t w = split_half2(fmaxf(fminf(nI - thr, kNoHit), -kNoHit));
             __syncwarp();
             if (CHI) W.op[lane].x = w;
             else W.op[2 * lane + 1].w = w;
@@ -600,7 +602,7 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
                         const ChiTerms t = chi_terms(X, S);
                         const float c = fmaf(D.f_c1, sl, D.f_c0);
                         const bool home = act && t.xy_ - share < kNoHit && fabsf(t.xs) + fabsf(t.ys) < kNoHit;
-                        nI = home ? t.xy_ - share : 2.f * kNoHit;
+                        nI = home ? t.xy_ - share : R<float>::inf();
                         // (y, x), (s, x) and (s, y) with the signs flipped, then the own terms
                         uint32_t yx[3], sx[3], sy[3];
 #pragma unroll
@@ -609,17 +611,17 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
                             sx[d] = home ? lo_lo(t.s[d], t.xy[d]) ^ kNegHalves : 0u;
                             sy[d] = home ? lo_lo(t.s[d], t.xy[d] >> 16) ^ kNegHalves : 0u;
                         }
-                        const uint32_t nf = home ? split_half2(t.ys + c) : 0u;
+                        const uint32_t nf = home ? split_half2(fminf(t.ys + c, kNoHit)) : 0u;
                         rows_of(make_uint4(yx[0], yx[1], yx[2], kOneOne), A);
                         rows_of(make_uint4(sx[0], sx[1], sx[2], kOneOne), A + 4);
                         rows_of(make_uint4(sy[0], sy[1], sy[2], 0u), A + 8);
                         rows_of(make_uint4(lo_lo(kOneOne, nf), hi_lo(kOneOne, nf >> 16), 0u, 0u), N + 4);
                         __syncwarp();
-                        W.op[lane] = make_uint4(0u, home ? split_half2(t.xs - c) : 0u, 0u, 0u);
+                        W.op[lane] = make_uint4(0u, home ? split_half2(fmaxf(t.xs - c, -kNoHit)) : 0u, 0u, 0u);
                     } else {
                         const PathTerms t = path_terms(X, S);
                         const bool home = act && t.N - share < kNoHit;
-                        nI = home ? t.N - share : 2.f * kNoHit;
+                        nI = home ? t.N - share : R<float>::inf();
                         const uint32_t mh01 = times2(t.mh01), mh2 = times2(t.mh2), ml01 = times2(t.ml01),
                                        ml2 = times2(t.ml2), h01 = times2(t.h01), h2 = times2(t.h2);
                         // words (0, 4 | 1, 5) and (2, 6 | 3, 7)

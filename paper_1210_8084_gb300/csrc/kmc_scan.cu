@@ -38,7 +38,7 @@ __device__ __forceinline__ int fixed_exponent(double m) {
 }
 
 // Frames, units and margins of the filtered search (derivation at the head of
-// kmc_filter.cuh) for a largest displacement s = v_max dt and a reach
+// kmc_filter.cuh) for a largest displacement s = v_max dt; the reach is
 // D = R + 2 s.  The frames are as wide as keeps the rounding margin of an
 // ordinary pair to about a tenth of what decides it: R^2 + |v_rel|^2 dt^2 / 4
 // with one filter (R counts little where the threshold falls to the closest
@@ -46,12 +46,10 @@ __device__ __forceinline__ int fixed_exponent(double m) {
 // for any width.
 // Computed in binary32 (one thread per instance, in the way of the step; binary64
 // took 7 us): every bound carries a factor of 1 + 2^-10, far above its rounding.
-__device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo, float s, float D) {
+__device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo, float s) {
     const float up = 1.f + 0x1p-10f, r3 = 1.7320508f * up;
-    const float R2 = (float)in.R2 * (1.f + 0x1p-20f), Rc = sqrtf(R2) * (1.f + 0x1p-20f), Re = in.sym ? Rc : 0.125f * Rc;
     s *= 1.f + 0x1p-20f;
-    D *= 1.f + 0x1p-20f;
-    float cmax = 0.f, lmax = 0.f, reach = 0.f;   // reach: largest separation of neighbouring c-bins, at most D
+    float cmax = 0.f, lmax = 0.f;
     float w[3];
     int image = 0;
     for (int d = 0; d < geo.dim; ++d) {
@@ -59,8 +57,16 @@ __device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo,
         const float L = (float)geo.L[d];
         cmax = fmaxf(cmax, fmaxf(fabsf((float)geo.lo[d]), fabsf((float)geo.hi[d])));
         lmax = fmaxf(lmax, L);
+    }
+    // a contact distance beyond 2^20 boxes lets every pair pass, as one of 2^20 boxes does
+    const float far = 0x1p20f * (lmax + s);
+    const float R2 = fminf((float)in.R2, far * far) * (1.f + 0x1p-20f), Rc = sqrtf(R2) * (1.f + 0x1p-20f),
+                Re = in.sym ? Rc : 0.125f * Rc;
+    const float D = (Rc + 2.f * s) * (1.f + 0x1p-20f);
+    float reach = 0.f;   // largest separation of neighbouring c-bins, at most D
+    for (int d = 0; d < geo.dim; ++d) {
         reach = fmaxf(reach, fminf(D, 2.f * (float)in.s[d] * w[d]));
-        if (geo.bc[d] == KMC_BC_PERIODIC && (geo.n[d] < 5 || D >= 0.499f * L)) image = 1;
+        if (geo.bc[d] == KMC_BC_PERIODIC && (geo.n[d] < 5 || D >= 0.499f * (float)geo.L[d])) image = 1;
     }
     const float aim = in.chi ? fminf(200.f * Rc, 400.f * s) : 46.f * sqrtf(Re * Re + s * s / 16.f);
     const float width = 2.f * (aim - reach - s);
@@ -149,7 +155,7 @@ __device__ void step_bookkeeping(InstDyn* dyn, const InstDev* inst, int n_inst, 
         for (int d = 0; d < geo.dim; ++d)
             if (geo.bc[d] == KMC_BC_PERIODIC && D * 1.001 >= 0.499 * geo.L[d]) dyn[i].p_image = 1;
         dyn[i].p_slack = (float)(0x1p-19 * D * D);
-        if (inst[i].search == kSearchFilter) filter_constants(dyn[i], inst[i], geo, (float)(vmax * dt), (float)D);
+        if (inst[i].search == kSearchFilter) filter_constants(dyn[i], inst[i], geo, (float)(vmax * dt));
     }
     if (threadIdx.x == 0 && bump) st->step += 1u;
 }
