@@ -399,7 +399,9 @@ SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms,
     I.close = passing > kPairsClose ? 1 : 0;
     if (h->precision == 64) {
         h->filter_chi = 1;
-        return search_costs64((double)h->n, cand, n_row);
+        SearchCosts c = search_costs64((double)h->n, cand, n_row);
+        if (!filter_fits(I, h->geo, dt0)) c.ps[kSearchFilter] = INFINITY;
+        return c;
     }
     bool wraps = false;   // with room for v_max to grow (InstDyn::p_image)
     for (int d = 0; d < h->dim; ++d) wraps = wraps || (h->geo.bc[d] == KMC_BC_PERIODIC && reach > 0.4 * h->geo.L[d]);
@@ -418,7 +420,7 @@ void choose_searches(kmc_handle* h, const std::vector<SearchCosts>& cost) {
         prune = prune || (I.prune && I.n > 0);
         n += I.n;
     }
-    unsigned best = 1u << kSearchFilter;
+    unsigned best = 1u << kSearchDirect;
     double least = INFINITY;
     for (unsigned set = 1; set < 8; ++set) {
         if ((prune || h->precision == 64) && (set & (1u << kSearchPairs))) continue;
@@ -839,7 +841,10 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
             costs.push_back(estimate_search(h, h->inst_h[i], vmax[i], sample[1] > 0.0 ? sqrt(sample[0] / sample[1]) : 0.0, occ[i]));
         }
         choose_searches(h, costs);
-        for (auto& I : h->inst_h) I.chi = h->filter_chi;
+        for (auto& I : h->inst_h) {
+            I.chi = h->filter_chi;
+            filter_lengths(I, h->geo);
+        }
         h->n_keys = (uint32_t)keys;
         h->cbin_moments = 1;
         for (const InstDev& I : h->inst_h)

@@ -74,6 +74,22 @@ __device__ __forceinline__ double frame_centre(const GeoT<double>& G, const Inst
     return G.lo[d] + 0.5 * (double)c2 * I.w[d];
 }
 
+// a speed in binary32, the largest number where it is out of range
+__device__ __forceinline__ float to_float_finite(float v) { return v; }
+__device__ __forceinline__ float to_float_finite(double v) { return __double2float_rz(v); }
+
+// A particle's path along one dimension in a frame of centre `ctr`: coordinate X and
+// displacement S in the frame's units; xf and sf the same for the swept boxes, `image`
+// lower.
+struct Path1 {
+    float X, S, xf, sf;
+};
+template <typename T>
+__device__ __forceinline__ Path1 path_in_frame(const InstDyn& D, T x, T v, T ctr, T image) {
+    const float vf = to_float_finite(v);
+    return Path1{(float)(x - ctr) * D.f_scale, vf * D.f_dts, (float)(x - image), vf * D.dtf};
+}
+
 // A particle's operands in a frame from its coordinates X and displacement S in
 // the frame's units, as a candidate (columns of B) or a home (rows of A), with its
 // own terms in two halves (high, low).  The product is of depth 16; lane 4 r + q of
@@ -175,19 +191,19 @@ __global__ void __launch_bounds__(kThreads) filter_prep_kernel(Bufs<T> b) {
         // sorted position by id, read by the move kernel to find a partner
         b.slot_of[I.p_off + (int64_t)tag_id(b, tag)] = (uint32_t)p;
         const T x[3] = {P.x, P.y, P.z}, v[3] = {Q.x, Q.y, Q.z};
-        const float sc = D.f_scale;
         float X[3] = {0.f, 0.f, 0.f}, S[3] = {0.f, 0.f, 0.f}, s2 = 0.f;
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
             int c, g;
             cell_and_search<T>(x[d], G.lo[d], G.inv[d], G.n[d], I.s[d], c, g);
             const int sh = D.f_shift[d];
-            X[d] = (float)(x[d] - frame_centre(G, I, D, d, (((g >> sh) * 2) << sh) + min(1 << sh, I.M[d]))) * sc;
-            const float s = (float)v[d] * D.dtf, xf = (float)x[d];
-            S[d] = s * sc;
+            const T ctr = frame_centre(G, I, D, d, (((g >> sh) * 2) << sh) + min(1 << sh, I.M[d]));
+            const Path1 w = path_in_frame(D, x[d], v[d], ctr, (T)0);
+            X[d] = w.X;
+            S[d] = w.S;
             s2 += S[d] * S[d];
-            lo[d] = fminf(xf, xf + s);
-            hi[d] = fmaxf(xf, xf + s);
+            lo[d] = fminf(w.xf, w.xf + w.sf);
+            hi[d] = fmaxf(w.xf, w.xf + w.sf);
         }
         const float sl = sqrtf(s2);
         const float share = fmaf(D.f_g1, sl, D.f_g0);   // this particle's share of the margin
@@ -277,9 +293,10 @@ struct FiltBest<float> {
     __device__ __forceinline__ void offer(bool pass, int i, float d2, uint32_t tag) {
         if (pass) atomicMin(&key[i], partner_key<float>(d2, tag));
     }
-    __device__ __forceinline__ bool distance2(int i, float& d2) const {
+    // distance of the closest candidate in the frame's units
+    __device__ __forceinline__ bool distance(int i, const InstDyn& D, float& d) const {
         const uint32_t o = (uint32_t)(key[i] >> 32);
-        d2 = __uint_as_float((o & 0x80000000u) ? (o ^ 0x80000000u) : ~o);
+        d = sqrtf(fmaxf(__uint_as_float((o & 0x80000000u) ? (o ^ 0x80000000u) : ~o), 0.f)) * D.f_scale;
         return o != 0xffffffffu;
     }
 };
@@ -300,8 +317,8 @@ struct FiltBest<double> {
             __syncwarp();
         }
     }
-    __device__ __forceinline__ bool distance2(int i, float& d) const {
-        d = (float)d2[i];
+    __device__ __forceinline__ bool distance(int i, const InstDyn& D, float& d) const {
+        d = sqrtf(fmaxf((float)d2[i], 0.f)) * D.f_scale;
         return id[i] != 0xffffffffu;
     }
 };
@@ -421,11 +438,8 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
         auto put_own = [&]() {
             float thr = D.f_thr;
             if (!sym) {
-                float d2;
-                if (W.best.distance2(lane, d2)) {
-                    d2 = fmaxf(d2, 0.f);
-                    thr = fminf(thr, fmaf(d2 * (1.f + 0x1p-20f), D.f_sc2, fmaf(D.f_rt, sqrtf(d2), D.f_slack)));
-                }
+                float d;   // distance of the closest candidate so far
+                if (W.best.distance(lane, D, d)) thr = fminf(thr, fmaf(d * (1.f + 0x1p-19f), d, fmaf(D.f_rt, d, D.f_slack)));
             }
             // (a contact distance beyond the frames' width: within binary16's range all the same)
             const uint32_t w = split_half2(fmaxf(fminf(nI - thr, kNoHit), -kNoHit));
@@ -560,7 +574,6 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
                 if (!built) {   // the homes in this frame
                     built = true;
                     images = images || w.kx != 0 || w.ky != 0 || w.kz != 0 || D.f_image != 0;
-                    const float sc = D.f_scale;
                     const int c2[3] = {w.cx2, DIM == 3 ? w.cy2 : w.cz2, w.cz2};
                     T ctr[3] = {(T)0, (T)0, (T)0};
 #pragma unroll
@@ -573,13 +586,13 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
                     const int kd[3] = {w.kx, DIM == 3 ? w.ky : w.kz, w.kz};
 #pragma unroll
                     for (int d = 0; d < DIM; ++d) {
-                        X[d] = (float)(x[d] - ctr[d]) * sc;
-                        const float s = (float)v[d] * D.dtf, xf = (float)(x[d] - (T)kd[d] * G.L[d]);
-                        S[d] = s * sc;
+                        const Path1 p = path_in_frame(D, x[d], v[d], ctr[d], (T)kd[d] * G.L[d]);
+                        X[d] = p.X;
+                        S[d] = p.S;
                         s2 += S[d] * S[d];
                         // widened by the contact distance and the rounding of the exact test
-                        lo[d] = act ? fminf(xf, xf + s) - D.f_box : R<float>::inf();
-                        hi[d] = act ? fmaxf(xf, xf + s) + D.f_box : -R<float>::inf();
+                        lo[d] = act ? fminf(p.xf, p.xf + p.sf) - D.f_box : R<float>::inf();
+                        hi[d] = act ? fmaxf(p.xf, p.xf + p.sf) + D.f_box : -R<float>::inf();
 #pragma unroll
                         for (int o = 1; o < 32; o <<= 1) {
                             lo[d] = fminf(lo[d], __shfl_xor_sync(kFull, lo[d], o));

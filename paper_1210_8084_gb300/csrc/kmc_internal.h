@@ -73,6 +73,11 @@ struct InstDev {
     int tile_rows;
     int tiles_per_x;     // ceil(M[1] / tile_rows)
     uint32_t tile_base;  // first tile of the instance in the staged launch
+    // Lengths for the filtered search's constants in units of 1 / f_unit, the power of two that
+    // puts the box's longest side in [1, 2): boxes of any size fit binary32 and binary16
+    float f_unit, f_len;    // f_unit and 1 / f_unit
+    float f_L[3], f_cw[3];  // box, search cell widths
+    float f_c, f_lmax, f_R; // largest coordinate, longest side, contact distance
 };
 
 // Per-instance quantities that change every step (written on the device).
@@ -86,16 +91,16 @@ struct InstDyn {
     int k[3];                       // search half-window in search cells
     int mom_e[3];                   // moment sums: fixed-point exponents of v, v^2 and W
     // filtered search (kmc_filter.cuh): frames of 2^f_shift search cells (at most all), coordinates
-    // in units of 1 / f_scale (a power of two); f_box a length, the other
-    // margins in the square of those units (f_g1, f_c1 per unit of displacement)
+    // in units of 1 / f_scale (a power of two); the margins in the square of those units (f_g1,
+    // f_c1, f_rt per unit of length)
     int f_shift[3];
     float f_w[3];                   // search cell widths (binary32)
     int f_image;                    // a window may hold a pair at more than half a periodic box
-    float f_scale, f_sc2;           // scale, scale^2
+    float f_scale, f_dts;           // the scale, scale x timestep
     float f_g0, f_g1;               // a particle's share of F's margin: f_g0 + f_g1 |s|
     float f_c0, f_c1;               // the same of the margin of a and f
     float f_thr;                    // threshold at the contact distance
-    float f_rt, f_slack;            // threshold at distance d: d^2 f_sc2 + f_rt d + f_slack
+    float f_rt, f_slack;            // threshold at distance d (in those units): d^2 + f_rt d + f_slack
     float f_box;                    // widening of a home's swept box
     // pair search (kmc_pairs.cuh)
     int p_image;                    // a pair may meet at half a periodic box or more
@@ -258,6 +263,35 @@ template <typename T>
 cudaError_t launch_dsmc(const Bufs<T>& b, cudaStream_t s);     // random-partner collisions per c-bin
 template <typename T>
 cudaError_t launch_cbin_hist(const Bufs<T>& b, uint32_t* hist, unsigned long long* vmax2, double* sample, cudaStream_t s);
+
+// Lengths of an instance for the filtered search (I.R2, I.w set).  A contact distance
+// beyond 2^20 boxes lets every pair pass, as one of 2^20 boxes does.
+inline void filter_lengths(InstDev& I, const Geo& g) {
+    double lmax = 0.0, cmax = 0.0;
+    for (int d = 0; d < g.dim; ++d) {
+        lmax = fmax(lmax, g.L[d]);
+        cmax = fmax(cmax, fmax(fabs(g.lo[d]), fabs(g.hi[d])));
+    }
+    const double unit = ldexp(1.0, -ilogb(lmax));
+    I.f_unit = (float)unit;
+    I.f_len = (float)ldexp(1.0, ilogb(lmax));
+    for (int d = 0; d < 3; ++d) {
+        I.f_L[d] = d < g.dim ? (float)(g.L[d] * unit) : 0.f;
+        I.f_cw[d] = d < g.dim ? (float)(I.w[d] * unit) : 0.f;
+    }
+    I.f_c = (float)(cmax * unit);
+    I.f_lmax = (float)(lmax * unit);
+    I.f_R = (float)fmin(sqrt(I.R2) * unit, 0x1p20);
+}
+
+// Whether a binary64 instance's lengths and timestep fit the filtered search, whose
+// operands and swept boxes are differences and products rounded to binary32 (their
+// squares must fit too).  Otherwise it takes one thread per particle.
+inline bool filter_fits(const InstDev& I, const Geo& g, double dt) {
+    double lmax = 0.0;
+    for (int d = 0; d < g.dim; ++d) lmax = fmax(lmax, g.L[d]);
+    return lmax > 0x1p-40 && lmax < 0x1p40 && dt > 0x1p-60 && dt < 0x1p60;
+}
 
 // Particles the buffers of a state of n hold: whole groups of 32, so that the filtered
 // search's operands of a last tile of 8, and that tile's box, lie inside them.

@@ -54,7 +54,12 @@ __device__ __forceinline__ uint32_t tag_of(double w) {
 
 // The instance table, passed by value (kernel parameters live with the launch,
 // so no host buffer has to outlive the call).
-__global__ void put_instance(InstDev* dst, InstDev I) { *dst = I; }
+static_assert(sizeof(InstDev) % sizeof(uint32_t) == 0, "whole words");
+__global__ void put_instance(InstDev* dst, InstDev I) {   // a word per thread
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(&I);
+    for (int i = threadIdx.x; i < (int)(sizeof(InstDev) / sizeof(uint32_t)); i += blockDim.x)
+        reinterpret_cast<uint32_t*>(dst)[i] = w[i];
+}
 
 // Closest candidate per particle (its tag is the low half of the partner
 // key; one instance, so tag = id), by id.
@@ -139,11 +144,13 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     const double n_row = (double)n / n_rows;
     I.search = n == 0 ? kSearchDirect
                : sizeof(T) == 8
-                   ? cheapest_search(search_costs64((double)n, cand, n_row), 1u << kSearchDirect | 1u << kSearchFilter)
+                   ? cheapest_search(search_costs64((double)n, cand, n_row),
+                                     1u << kSearchDirect | (filter_fits(I, g, I.dt) ? 1u << kSearchFilter : 0u))
                    : cheapest_search(search_costs(g.dim, split, wraps, (double)n, cand, I.sym ? 0.25 * near : 0.1 * cand, passing,
                                                     rows, n_row), 7u);
     I.close = passing > kPairsClose ? 1 : 0;
     I.chi = sizeof(T) == 8 ? 1 : 0;
+    filter_lengths(I, g);
     Bufs<T> b{};
     b.n = n;
     b.n_inst = 1;
@@ -180,7 +187,7 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     b.id_bits = 32;
     b.id_mask = 0xffffffffu;
     // the array keeps the last call's contents: clear what must start at zero
-    put_instance<<<1, 1, 0, s>>>((InstDev*)b.inst, I);
+    put_instance<<<1, 64, 0, s>>>((InstDev*)b.inst, I);
     if (cudaGetLastError() != cudaSuccess) return KMC_ECUDA;
     if (cudaMemsetAsync(b.st, 0, sizeof(DevState), s) != cudaSuccess) return KMC_ECUDA;
     if (cudaMemsetAsync(b.dyn, 0, sizeof(InstDyn), s) != cudaSuccess) return KMC_ECUDA;

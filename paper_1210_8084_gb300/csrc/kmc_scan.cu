@@ -45,28 +45,21 @@ __device__ __forceinline__ int fixed_exponent(double m) {
 // candidate so far: R / 8), R and |v_rel| dt with three.  Every bound below holds
 // for any width.
 // Computed in binary32 (one thread per instance, in the way of the step; binary64
-// took 7 us): every bound carries a factor of 1 + 2^-10, far above its rounding.
-__device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo, float s) {
+// took 7 us): every bound carries a factor of 1 + 2^-10, far above its rounding.  Lengths
+// are in units of f_len, or of s where that is longer, so nothing leaves the range.
+__device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo, double displacement) {
     const float up = 1.f + 0x1p-10f, r3 = 1.7320508f * up;
-    s *= 1.f + 0x1p-20f;
-    float cmax = 0.f, lmax = 0.f;
-    float w[3];
+    float s = (float)fmin(displacement * (double)in.f_unit, 0x1p100) * (1.f + 0x1p-20f);
+    const float z = s > 1.f ? __int_as_float((127 - ilogbf(s)) << 23) : 1.f;
+    s *= z;
+    const float Rc = in.f_R * z * (1.f + 0x1p-20f), R2 = Rc * Rc * (1.f + 0x1p-20f), Re = in.sym ? Rc : 0.125f * Rc;
+    const float D = (Rc + 2.f * s) * (1.f + 0x1p-20f), cmax = in.f_c * z, lmax = in.f_lmax * z;
+    float w[3], reach = 0.f;   // reach: largest separation of neighbouring c-bins, at most D
     int image = 0;
     for (int d = 0; d < geo.dim; ++d) {
-        w[d] = (float)in.w[d];
-        const float L = (float)geo.L[d];
-        cmax = fmaxf(cmax, fmaxf(fabsf((float)geo.lo[d]), fabsf((float)geo.hi[d])));
-        lmax = fmaxf(lmax, L);
-    }
-    // a contact distance beyond 2^20 boxes lets every pair pass, as one of 2^20 boxes does
-    const float far = 0x1p20f * (lmax + s);
-    const float R2 = fminf((float)in.R2, far * far) * (1.f + 0x1p-20f), Rc = sqrtf(R2) * (1.f + 0x1p-20f),
-                Re = in.sym ? Rc : 0.125f * Rc;
-    const float D = (Rc + 2.f * s) * (1.f + 0x1p-20f);
-    float reach = 0.f;   // largest separation of neighbouring c-bins, at most D
-    for (int d = 0; d < geo.dim; ++d) {
+        w[d] = in.f_cw[d] * z;
         reach = fmaxf(reach, fminf(D, 2.f * (float)in.s[d] * w[d]));
-        if (geo.bc[d] == KMC_BC_PERIODIC && (geo.n[d] < 5 || D >= 0.499f * (float)geo.L[d])) image = 1;
+        if (geo.bc[d] == KMC_BC_PERIODIC && (geo.n[d] < 5 || D >= 0.499f * z * in.f_L[d])) image = 1;
     }
     const float aim = in.chi ? fminf(200.f * Rc, 400.f * s) : 46.f * sqrtf(Re * Re + s * s / 16.f);
     const float width = 2.f * (aim - reach - s);
@@ -77,7 +70,7 @@ __device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo,
         if (d < geo.dim) {
             while ((1 << sh) < in.M[d] && (float)min(2 << sh, in.M[d]) * w[d] <= width) ++sh;
             half = fmaxf(half, 0.5f * (float)min(1 << sh, in.M[d]) * w[d]);
-            dy.f_w[d] = w[d];
+            dy.f_w[d] = (float)in.w[d];
         }
         dy.f_shift[d] = sh;
     }
@@ -104,12 +97,18 @@ __device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo,
         dy.f_c0 = dy.f_c1 = 0.f;
     }
     dy.f_image = image;
-    dy.f_scale = sc;
-    dy.f_sc2 = sc2;
-    dy.f_rt = 2.f * r3 * E * sc2;
+    dy.f_scale = sc * z * in.f_unit;
+    dy.f_dts = dy.f_scale * dy.dtf;
+    dy.f_rt = 2.f * r3 * E * sc;
     dy.f_slack = slack * up * sc2;
     dy.f_thr = (R2 + 2.f * r3 * E * Rc + slack * up) * sc2;
-    dy.f_box = Rc * up + 0x1p-9f * D + 0x1p-18f * (cmax + lmax);
+    dy.f_box = (Rc * up + 0x1p-9f * D + 0x1p-18f * (cmax + lmax)) / z * in.f_len;
+    // speeds or timesteps out of binary32's range (binary64 states set later): every pair passes
+    if (!(displacement < 0x1p100 * in.f_len && dy.dt > 0x1p-100 && dy.dt < 0x1p100)) {
+        dy.f_scale = dy.f_dts = dy.f_g0 = dy.f_g1 = dy.f_c1 = dy.f_rt = 0.f;
+        dy.f_c0 = dy.f_thr = dy.f_slack = 1.f;
+        dy.f_box = __int_as_float(0x7f800000);
+    }
 }
 
 __device__ void step_bookkeeping(InstDyn* dyn, const InstDev* inst, int n_inst, DevState* st, const Geo& geo,
@@ -155,7 +154,7 @@ __device__ void step_bookkeeping(InstDyn* dyn, const InstDev* inst, int n_inst, 
         for (int d = 0; d < geo.dim; ++d)
             if (geo.bc[d] == KMC_BC_PERIODIC && D * 1.001 >= 0.499 * geo.L[d]) dyn[i].p_image = 1;
         dyn[i].p_slack = (float)(0x1p-19 * D * D);
-        if (inst[i].search == kSearchFilter) filter_constants(dyn[i], inst[i], geo, (float)(vmax * dt));
+        if (inst[i].search == kSearchFilter) filter_constants(dyn[i], inst[i], geo, vmax * dt);
     }
     if (threadIdx.x == 0 && bump) st->step += 1u;
 }
