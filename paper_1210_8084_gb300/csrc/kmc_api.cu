@@ -843,7 +843,7 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         choose_searches(h, costs);
         for (auto& I : h->inst_h) {
             I.chi = h->filter_chi;
-            filter_lengths(I, h->geo);
+            filter_lengths(I, h->geo, h->precision == 64);
         }
         h->n_keys = (uint32_t)keys;
         h->cbin_moments = 1;

@@ -74,20 +74,19 @@ __device__ __forceinline__ double frame_centre(const GeoT<double>& G, const Inst
     return G.lo[d] + 0.5 * (double)c2 * I.w[d];
 }
 
-// a speed in binary32, the largest number where it is out of range
-__device__ __forceinline__ float to_float_finite(float v) { return v; }
-__device__ __forceinline__ float to_float_finite(double v) { return __double2float_rz(v); }
-
 // A particle's path along one dimension in a frame of centre `ctr`: coordinate X and
-// displacement S in the frame's units; xf and sf the same for the swept boxes, `image`
-// lower.
+// displacement S in the frame's units; xf and sf the same for the swept boxes.  Those
+// are in binary32's coordinates, `image` lower; in binary64 from the low wall on, the
+// centre at `off` (a box far from the origin would lose its digits).
 struct Path1 {
     float X, S, xf, sf;
 };
-template <typename T>
-__device__ __forceinline__ Path1 path_in_frame(const InstDyn& D, T x, T v, T ctr, T image) {
-    const float vf = to_float_finite(v);
-    return Path1{(float)(x - ctr) * D.f_scale, vf * D.f_dts, (float)(x - image), vf * D.dtf};
+__device__ __forceinline__ Path1 path_in_frame(const InstDyn& D, float x, float v, float ctr, float image, float) {
+    return Path1{(x - ctr) * D.f_scale, v * D.f_dts, x - image, v * D.dtf};
+}
+__device__ __forceinline__ Path1 path_in_frame(const InstDyn& D, double x, double v, double ctr, double, float off) {
+    const float xc = (float)(x - ctr), vf = __double2float_rz(v);   // rz: a speed out of range stays finite
+    return Path1{xc * D.f_scale, vf * D.f_dts, xc + off, vf * D.dtf};
 }
 
 // A particle's operands in a frame from its coordinates X and displacement S in
@@ -197,8 +196,8 @@ __global__ void __launch_bounds__(kThreads) filter_prep_kernel(Bufs<T> b) {
             int c, g;
             cell_and_search<T>(x[d], G.lo[d], G.inv[d], G.n[d], I.s[d], c, g);
             const int sh = D.f_shift[d];
-            const T ctr = frame_centre(G, I, D, d, (((g >> sh) * 2) << sh) + min(1 << sh, I.M[d]));
-            const Path1 w = path_in_frame(D, x[d], v[d], ctr, (T)0);
+            const int c2 = (((g >> sh) * 2) << sh) + min(1 << sh, I.M[d]);
+            const Path1 w = path_in_frame(D, x[d], v[d], frame_centre(G, I, D, d, c2), (T)0, 0.5f * (float)c2 * D.f_w[d]);
             X[d] = w.X;
             S[d] = w.S;
             s2 += S[d] * S[d];
@@ -586,7 +585,8 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
                     const int kd[3] = {w.kx, DIM == 3 ? w.ky : w.kz, w.kz};
 #pragma unroll
                     for (int d = 0; d < DIM; ++d) {
-                        const Path1 p = path_in_frame(D, x[d], v[d], ctr[d], (T)kd[d] * G.L[d]);
+                        const Path1 p = path_in_frame(D, x[d], v[d], ctr[d], (T)kd[d] * G.L[d],
+                                                      0.5f * (float)(c2[d] - 2 * kd[d] * I.M[d]) * D.f_w[d]);
                         X[d] = p.X;
                         S[d] = p.S;
                         s2 += S[d] * S[d];

@@ -76,6 +76,7 @@ struct InstDev {
     // Lengths for the filtered search's constants in units of 1 / f_unit, the power of two that
     // puts the box's longest side in [1, 2): boxes of any size fit binary32 and binary16
     float f_unit, f_len;    // f_unit and 1 / f_unit
+    int f64;                // binary64 state
     float f_L[3], f_cw[3];  // box, search cell widths
     float f_c, f_lmax, f_R; // largest coordinate, longest side, contact distance
 };
@@ -266,7 +267,8 @@ cudaError_t launch_cbin_hist(const Bufs<T>& b, uint32_t* hist, unsigned long lon
 
 // Lengths of an instance for the filtered search (I.R2, I.w set).  A contact distance
 // beyond 2^20 boxes lets every pair pass, as one of 2^20 boxes does.
-inline void filter_lengths(InstDev& I, const Geo& g) {
+inline void filter_lengths(InstDev& I, const Geo& g, bool binary64) {
+    I.f64 = binary64;
     double lmax = 0.0, cmax = 0.0;
     for (int d = 0; d < g.dim; ++d) {
         lmax = fmax(lmax, g.L[d]);

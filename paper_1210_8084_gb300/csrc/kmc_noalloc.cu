@@ -150,7 +150,7 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
                                                     rows, n_row), 7u);
     I.close = passing > kPairsClose ? 1 : 0;
     I.chi = sizeof(T) == 8 ? 1 : 0;
-    filter_lengths(I, g);
+    filter_lengths(I, g, sizeof(T) == 8);
     Bufs<T> b{};
     b.n = n;
     b.n_inst = 1;

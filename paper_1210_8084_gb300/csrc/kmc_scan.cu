@@ -77,7 +77,10 @@ __device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo,
     // largest coordinate of a candidate in its frame and of a home that may pair with it
     const float X = (half + reach + s) * up;
     const float sc = __int_as_float((127 + 4 - ilogbf(X)) << 23), sc2 = sc * sc;   // X sc in [16, 32)
-    const float e32 = 0x1p-20f * (cmax + lmax + s), tiny = 0x1p-23f / sc;
+    // rounding of the coordinates and frame centres; binary64 rounds to binary32 after it has
+    // taken the difference from the centre (the boxes' coordinates: and added the centre's)
+    const float far = in.f64 ? 0x1p-50f * (cmax + lmax) : 0x1p-20f * (cmax + lmax);
+    const float e32 = far + 0x1p-20f * (in.f64 ? X + s : s), tiny = 0x1p-23f / sc;
     float slack = 0x1p-17f * D * D + 0x1p-18f * 12.f * X * X;
     float E;   // error of a separation component that |r0| + |r1| (three filters) or |dm| (one) multiplies
     if (in.chi) {
@@ -102,7 +105,7 @@ __device__ void filter_constants(InstDyn& dy, const InstDev& in, const Geo& geo,
     dy.f_rt = 2.f * r3 * E * sc;
     dy.f_slack = slack * up * sc2;
     dy.f_thr = (R2 + 2.f * r3 * E * Rc + slack * up) * sc2;
-    dy.f_box = (Rc * up + 0x1p-9f * D + 0x1p-18f * (cmax + lmax)) / z * in.f_len;
+    dy.f_box = (Rc * up + 0x1p-9f * D + 4.f * far + (in.f64 ? 0x1p-18f * lmax : 0.f)) / z * in.f_len;
     // speeds or timesteps out of binary32's range (binary64 states set later): every pair passes
     if (!(displacement < 0x1p100 * in.f_len && dy.dt > 0x1p-100 && dy.dt < 0x1p100)) {
         dy.f_scale = dy.f_dts = dy.f_g0 = dy.f_g1 = dy.f_c1 = dy.f_rt = 0.f;

@@ -116,3 +116,26 @@ def test_partner_call_in_other_units(prec, unit):
         out.append(best.cpu().numpy())
     assert (out[0] >= 0).mean() > 0.3
     assert np.array_equal(*out)
+
+
+@pytest.mark.parametrize("offset", [1e3, 1e6, 1e9])
+def test_binary64_box_far_from_the_origin(offset):
+    """The pairs of one thread per particle, and (the margins do not grow with the offset) about the
+    search's time at the origin: bounds of binary32 coordinates let nearly every pair pass from 10^6 on."""
+    import paper_1210_8084_gb300 as k
+    from paper_1210_8084_gb300 import inputs
+    n, bc = 200_000, (WALL, PER, PER)
+    ms, out = [], []
+    for off, flags in ((0.0, 0), (offset, 0), (offset, k.KMC_FLAG_NO_TILE_SEARCH)):
+        lo, hi = (off,) * 3, (off + 1,) * 3
+        pos, vel = inputs.cast_state(*inputs.sod_tube(n, seed=4, lo=lo, hi=hi, split=off + 0.5), np.float64, lo, hi, bc)
+        sim = k.Simulation(k.make_config(dim_pos=3, n_cells=(200, 1, 1), lo=lo, hi=hi, bc=bc, lam=1e-3, dt=1e-3, seed=3,
+                                         precision=64, flags=flags | k.KMC_FLAG_RECORD), pos, vel)
+        assert sim.search()[0] == (k.KMC_SEARCH_PARTICLE if flags else k.KMC_SEARCH_FILTER)
+        ms.append(min(sim.step_profiled(1)["search"] for _ in range(5)))
+        out.append((*sim.partners(), *sim.state()))
+        sim.close()
+    assert (out[1][1] >= 0).mean() > 0.1
+    for a, b in zip(out[1], out[2]):
+        assert np.array_equal(a, b)
+    assert ms[1] < 1.5 * ms[0], ms
