@@ -310,10 +310,14 @@ inline int filter_split(int64_t n, int sms) {
 }
 
 // Counting-sort scatter of large cells (rank_cells_kernel): launches of it for a
-// state of n particles over n_keys search cells.
-constexpr uint32_t kRankMin = 64;        // cells up to this many particles: the moving pass counts
+// state of n particles over n_keys search cells.  Counting a cell's tags in the moving
+// pass, and ranking them by a block, both scatter passes of 4M particles, ms, by
+// particles per cell: 117 0.121 / 0.17, 169 0.139 / 0.15, 200 0.164 / 0.14, 400 0.254 / 0.12
+// (64M: 40 1.40 / 2.47, 64 1.57 / 2.98).  A launch costs each cell it leaves alone 0.5 ns, so
+// it is made where a mean cell is nearly large enough.
+constexpr uint32_t kRankMin = 192;       // cells up to this many particles: the moving pass counts
 constexpr int kRankCap = 4096;           // the first launch's largest cell (32 KiB of shared memory)
-constexpr int64_t kRankMean = 24;        // mean particles per cell from which the first launch runs
+constexpr int64_t kRankMean = 160;       // mean particles per cell from which the first launch runs
 constexpr int64_t kRankMeanLarge = 1024; // and from which the second runs, for cells up to kCanonMax
 inline int rank_launches(int64_t n, uint32_t n_keys) {
     const int64_t mean = n_keys > 0 ? n / (int64_t)n_keys : 0;
