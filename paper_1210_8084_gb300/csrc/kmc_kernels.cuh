@@ -2625,17 +2625,21 @@ __device__ __forceinline__ uint32_t tags_below(const uint32_t* __restrict__ t, u
 // in N).  The ids, spread over the instance's range, go to CAP / 2 buckets of
 // equal id range (a count, its prefix sums, a placement); a tag's rank is its
 // bucket's start plus the lower ids among the bucket's, about two for ids without
-// order (any order is right, a narrow range of ids only slower).  Both scatter
-// passes with this kernel, GB300: 64M particles in 262,144 cells (quadrants) 5.16 ->
-// 2.36 ms, 4M in 2000 cells 1.96 -> 0.12 ms.
+// order.  Where one bucket gets many (a state generated cell by cell: a cell's ids are
+// a narrow range), the buckets divide the cell's own range, and the tags are placed
+// themselves, to be compared four per load where a few far ids still crowd the
+// others.  Both scatter passes with this kernel, GB300, ms: 64M particles in 262,144 cells
+// (quadrants) 5.16 -> 2.36; 4M in 2000 cells 0.94 -> 0.11, with ids in cell order 0.94 ->
+// 0.12 (1.39 with the instance's range alone), the same but four far ids per cell 0.63.
 template <typename T, int CAP, int TPB>
 __global__ void __launch_bounds__(TPB) rank_cells_kernel(Bufs<T> b, uint32_t above) {
     constexpr int NB = CAP / 2, PER = NB / TPB;
-    extern __shared__ uint32_t rank_smem[];
+    constexpr uint32_t kCrowd = 32;   // a bucket of ids without order holds about two
+    extern __shared__ __align__(16) uint32_t rank_smem[];
     uint32_t* tg = rank_smem;                                                   // the cell's tags
     uint32_t* cnt = tg + CAP;                                                   // buckets
     unsigned short* idx = reinterpret_cast<unsigned short*>(cnt + NB);          // slots by bucket
-    __shared__ uint32_t wsum[TPB / 32];
+    __shared__ uint32_t wsum[TPB / 32], wmin[TPB / 32];
     const uint32_t kc = blockIdx.x;
     const uint32_t s0 = b.start[kc], s1 = b.start[kc + 1];
     const uint32_t N = s1 - s0;
@@ -2646,8 +2650,9 @@ __global__ void __launch_bounds__(TPB) rank_cells_kernel(Bufs<T> b, uint32_t abo
         if (b.inst[mid].key_base <= kc) lo = mid;
         else hi = mid - 1;
     }
-    const float scale = (float)NB / (float)b.inst[lo].n;
-    auto bucket = [&](uint32_t tag) { return min(NB - 1, (int)((float)tag_id(b, tag) * scale)); };
+    float scale = (float)NB / (float)b.inst[lo].n;
+    uint32_t base = 0u;
+    auto bucket = [&](uint32_t tag) { return min(NB - 1, (int)((float)(tag_id(b, tag) - base) * scale)); };
     uint32_t* tags = b.slot_of + s0;
     const int t = threadIdx.x;
     for (int i = t; i < NB; i += TPB) cnt[i] = 0u;
@@ -2658,11 +2663,43 @@ __global__ void __launch_bounds__(TPB) rank_cells_kernel(Bufs<T> b, uint32_t abo
         atomicAdd(&cnt[bucket(tag)], 1u);
     }
     __syncthreads();
-    uint32_t own[PER], sum = 0u;   // exclusive prefix sums of the counts
+    uint32_t own[PER], sum, most;   // exclusive prefix sums of the counts, the largest count
+    auto sums = [&]() {
+        sum = most = 0u;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        own[j] = sum;
-        sum += cnt[t * PER + j];
+        for (int j = 0; j < PER; ++j) {
+            const uint32_t c = cnt[t * PER + j];
+            own[j] = sum;
+            sum += c;
+            most = max(most, c);
+        }
+    };
+    sums();
+    const bool crowded = __syncthreads_or(most > kCrowd);
+    if (crowded) {   // count again over the cell's own range
+        uint32_t mn = 0xffffffffu, mx = 0u;
+        for (uint32_t i = t; i < N; i += TPB) {
+            const uint32_t id = tag_id(b, tg[i]);
+            mn = min(mn, id);
+            mx = max(mx, id);
+        }
+        mn = __reduce_min_sync(kFull, mn);
+        mx = __reduce_max_sync(kFull, mx);
+        if (lane_id() == 0) {
+            wmin[t >> 5] = mn;
+            wsum[t >> 5] = mx;
+        }
+        for (int i = t; i < NB; i += TPB) cnt[i] = 0u;
+        __syncthreads();
+        for (int w = 0; w < TPB / 32; ++w) {
+            mn = min(mn, wmin[w]);
+            mx = max(mx, wsum[w]);
+        }
+        base = mn;
+        scale = (float)NB / ((float)(mx - mn) + 1.f);
+        for (uint32_t i = t; i < N; i += TPB) atomicAdd(&cnt[bucket(tg[i])], 1u);
+        __syncthreads();
+        sums();
     }
     uint32_t inc = sum;
 #pragma unroll
@@ -2677,12 +2714,24 @@ __global__ void __launch_bounds__(TPB) rank_cells_kernel(Bufs<T> b, uint32_t abo
 #pragma unroll
     for (int j = 0; j < PER; ++j) cnt[t * PER + j] = before + own[j];
     __syncthreads();
-    for (uint32_t i = t; i < N; i += TPB) idx[atomicAdd(&cnt[bucket(tg[i])], 1u)] = (unsigned short)i;
+    if (crowded) {
+        for (uint32_t i = t; i < N; i += TPB) {
+            const uint32_t tag = tags[i], at = atomicAdd(&cnt[bucket(tag)], 1u);
+            tg[at] = tag;
+            idx[at] = (unsigned short)i;
+        }
+    } else {
+        for (uint32_t i = t; i < N; i += TPB) idx[atomicAdd(&cnt[bucket(tg[i])], 1u)] = (unsigned short)i;
+    }
     __syncthreads();   // cnt[k] is now the end of bucket k
     for (uint32_t i = t; i < N; i += TPB) {
         const uint32_t tag = tg[i];
         const int k = bucket(tag);
         const uint32_t q0 = k > 0 ? cnt[k - 1] : 0u, q1 = cnt[k];
+        if (crowded) {
+            tags[idx[i]] = q0 + tags_below(tg, q0, q1, tag);
+            continue;
+        }
         uint32_t r = q0;
         for (uint32_t q = q0; q < q1; ++q) r += tg[idx[q]] < tag ? 1u : 0u;
         tags[i] = r;

@@ -32,6 +32,34 @@ def _cells(order, cells, counts, seed=2):
     return cell
 
 
+@pytest.mark.parametrize("order", ["mixed", "by_cell", "few_far", "parts"])
+@pytest.mark.parametrize("cells,counts", [(3, [192, 193, 300]), (40, 500), (5, [4096, 700, 0, 4097, 2000]), (3, [16384, 16383, 9000])],
+                         ids=str)
+def test_order_in_cells(cells, counts, order):
+    import paper_1210_8084_gb300 as k
+    cell = _cells(order, cells, counts)
+    n = len(cell)
+    sim = _sim(k, cells, cell)
+    perm = sim.perm()
+    where = sim.cell_keys()[perm]
+    assert np.array_equal(np.sort(perm), np.arange(n))
+    assert np.all(np.diff(where) >= 0)
+    for c in range(cells):
+        assert np.all(np.diff(perm[where == c]) > 0) or np.count_nonzero(where == c) > 16384
+    sim.close()
+
+
+def test_ids_in_cell_order_take_no_longer():
+    """A state generated cell by cell: a cell's ids are a narrow range of the instance's."""
+    import paper_1210_8084_gb300 as k
+    ms = {}
+    for order in ("mixed", "by_cell"):
+        sim = _sim(k, 2000, _cells(order, 2000, 2000))
+        ms[order] = min(sim.step_profiled(1)["scatter"] for _ in range(5))
+        sim.close()
+    assert ms["by_cell"] < 2.0 * ms["mixed"], ms
+
+
 @pytest.mark.parametrize("mean,launches", [(40, 0), (100, 0), (200, 1), (2000, 2)])
 def test_small_cells_are_not_ranked(mean, launches):
     """Cells of less than some two hundred particles are put in order by the moving pass."""
