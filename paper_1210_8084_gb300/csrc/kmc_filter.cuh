@@ -551,8 +551,7 @@ __global__ void __launch_bounds__(WARPS * 32, (sizeof(T) == 8 ? 16 : CHI ? 24 : 
                         if (sym) q0 = max(q0, p0 + first + 1);
                     }
                 }
-                const int tile0 = q0 / kFiltTile;
-                const int cnt = q1 > q0 ? (q1 + kFiltTile - 1) / kFiltTile - tile0 : 0;
+                const int tile0 = q0 / kFiltTile, cnt = pieces_touched(q0, q1, kFiltTile);
                 incl = cnt;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {

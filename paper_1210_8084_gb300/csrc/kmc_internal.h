@@ -295,6 +295,20 @@ inline bool filter_fits(const InstDev& I, const Geo& g, double dt) {
     return lmax > 0x1p-40 && lmax < 0x1p40 && dt > 0x1p-60 && dt < 0x1p60;
 }
 
+#ifdef __CUDACC__
+#define KMC_HOST_DEVICE __host__ __device__
+#else
+#define KMC_HOST_DEVICE
+#endif
+// Pieces of `size` positions that positions [q0, q1) touch (counted from position 0) and
+// that they fill (counted from q0).  Positions go up to 2^31 - 2: nothing is rounded up past them.
+KMC_HOST_DEVICE inline int32_t pieces_touched(int32_t q0, int32_t q1, int32_t size) {
+    return q1 > q0 ? (q1 - 1) / size - q0 / size + 1 : 0;
+}
+KMC_HOST_DEVICE inline int32_t pieces_filled(int32_t q0, int32_t q1, int32_t size) {
+    return q1 > q0 ? (q1 - q0 - 1) / size + 1 : 0;
+}
+
 // Particles the buffers of a state of n hold: whole groups of 32, so that the filtered
 // search's operands of a last tile of 8, and that tile's box, lie inside them.
 inline size_t buffer_rows(int64_t n) { return ((size_t)(n > 0 ? n : 1) + 31) / 32 * 32; }

@@ -136,7 +136,9 @@ __global__ void __launch_bounds__(32, kPairsBlocks) pairs_search_kernel(Bufs<flo
                                      DIM == 3 ? (float)(1 - (int)(cd >> 2 & 3u)) * G.L[1] : (float)(1 - (int)(cd >> 4 & 3u)) * G.L[1],
                                      DIM == 3 ? (float)(1 - (int)(cd >> 4 & 3u)) * G.L[2] : 0.f};
                 const bool shifted = sh[0] != 0.f || sh[1] != 0.f || sh[2] != 0.f;
-                for (int32_t base = a0; base < a1; base += kPairsChunk) {
+                const int32_t chunks = pieces_filled(a0, a1, kPairsChunk);
+                for (int32_t chunk = 0; chunk < chunks; ++chunk) {
+                    const int32_t base = a0 + chunk * kPairsChunk;
                     const int n = min(kPairsChunk, a1 - base);
                     __syncwarp();
                     // a pair farther than both of its particles' closest so far is no pair
