@@ -137,8 +137,9 @@ typedef struct kmc_config {
     double occupancy_target; /* automatic subdivision: particles per search cell aimed at (0 = 0.5) */
     int flags;          /* KMC_FLAG_* */
     double radial_center[3]; /* centre of the radial velocity moment (KMC_MOM_RADIAL), finite */
-    int tile_threads;   /* the three: not 0 asks for one block per c-bin where search cells are the c-bins
-                         * (or, pruned, their halves).  Threads per block, a multiple of 32 from 64 to
+    int tile_threads;   /* the three: a value that is not the default (0, or what kmc_get_info reports for 0)
+                         * asks for one block per c-bin where search cells are the c-bins (or, pruned,
+                         * their halves).  Threads per block, a multiple of 32 from 64 to
                          * 256 (0 = 256); speed only, never results */
     int tile_cap;       /* the same: candidates staged in shared memory at once, even, 64 ... 6144 in
                          * binary32, 64 ... 3072 in binary64 (0 = 1536 / 768, 48 KiB); speed only */

@@ -263,6 +263,13 @@ int check_device_error(kmc_handle* h) {
     return KMC_OK;
 }
 
+// Whether the configuration's tile parameters ask for a block per c-bin: any value that
+// is not the default (0, or what kmc_get_info reports for 0).
+bool asks_for_tiles(const kmc_config& c) {
+    const bool cap = c.tile_cap == 0 || (c.precision == 64 ? c.tile_cap == 768 : c.tile_cap == 1536 || c.tile_cap == kPrunedCap);
+    return !((c.tile_threads == 0 || c.tile_threads == 256) && cap && (c.tile_split == 0 || c.tile_split == 1));
+}
+
 // Search-grid subdivision of instance i: cells of width >= D' (so the first
 // step searches +-1 cell) and about `target` particles per cell in the
 // densest c-bin, capped so the key count stays within a few times N.
@@ -345,7 +352,7 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
             // 2-D, (2, 2) and here: 20 per c-bin 1.29 -> 1.15, 125 3.38 -> 3.12, 400 8.03 ->
             // 7.80.  Small instances keep half c-bins, the grid that callers of
             // kmc_get_info have seen for them (20 % of a 0.3 ms step at 60,000).
-            if (I.n >= kFineRows && h->cfg.tile_threads == 0 && h->cfg.tile_cap == 0 && h->cfg.tile_split == 0) {
+            if (I.n >= kFineRows && !asks_for_tiles(h->cfg)) {
                 const double mean = (double)I.n / (double)h->bins_per_inst;
                 const int across = h->dim == 3 && mean > 64.0 ? 2 : 1;
                 for (int d = 0; d + 1 < h->dim; ++d) s[d] = across;
@@ -865,7 +872,7 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         for (const InstDev& I : h->inst_h) tile_grid = tile_grid || (I.s[0] == 1 && I.s[1] == 1 && I.s[2] == 1) || I.prune;
         const bool choose = !dsmc && n > 0 &&
                             !(h->cfg.flags & (KMC_FLAG_NO_TILE_SEARCH | KMC_FLAG_STAGED_SEARCH | KMC_FLAG_NO_TILE_PRUNE)) &&
-                            !(tile_grid && (h->cfg.tile_threads > 0 || h->cfg.tile_cap > 0 || h->cfg.tile_split > 0));
+                            !(tile_grid && asks_for_tiles(h->cfg));
         h->filtered = h->paired = 0;
         int64_t open = 0, close = 0;   // particles of pair-searched instances
         for (auto& I : h->inst_h) {
