@@ -163,6 +163,8 @@ KERNEL_SEGMENTS = {
 }
 
 
+# kernel by KMC_SEARCH_* of the handle's first instance
+SEARCH_KERNELS = ("search", "filter_search", "pairs_search", "tile_search", "tile_pruned", "search_staged")
 KERNEL_FILES = {"filter_search": "kmc_filter.cuh", "pairs_search": "kmc_pairs.cuh"}
 
 
@@ -250,6 +252,7 @@ def run_device(k, w, seed, steps, warmup, stream, occ=0.0, clocks=None, barrier=
                         tile_split=tile[2])
     sim = k.Simulation(cfg, pos, vel)
     info = sim.info()
+    search = sim.search()[0]
     e_start = sim.moments()[2][0, 1]
     sim.step_profiled(warmup, want_moments=1)
     if barrier:
@@ -266,7 +269,7 @@ def run_device(k, w, seed, steps, warmup, stream, occ=0.0, clocks=None, barrier=
     tests = (sim.tile_tests() - tests0) / (w["n"] * steps) if info.tile_prune and info.n_search_cells else None
     raw, der, glob = sim.moments()
     out = dict(prof=prof, info=info, clocks=clk, pairs=float(glob[0, 6]), e_start=float(e_start),
-               e_end=float(glob[0, 1]), cand=sim.window_size(), cfg=cfg, pos=pos, vel=vel, tile_tests=tests)
+               e_end=float(glob[0, 1]), cand=sim.window_size(), cfg=cfg, pos=pos, vel=vel, tile_tests=tests, search=search)
     sim.close()
     torch.cuda.synchronize()
     return out
@@ -279,9 +282,9 @@ def roofline_of(w, r, steps, n_sm, peaks, peak_src, workload):
     dom = max(("search", "tile", "move", "scan", "scatter", "moments"), key=lambda p: phases[p])
     t_dom = phases[dom] * 1e-3
     frac_paired = 2 * r["pairs"] / n
-    # instances that skip candidates out of reach: the filtered search, or the pruned tile search where asked for
+    # the search the handle took (kmc_get_search); instances that skip candidates out of reach count their tests
     pruned = dom in ("search", "tile") and r.get("tile_tests") is not None
-    kernel = {"search": "filter_search" if pruned else "search", "tile": "tile_pruned" if pruned else "tile_search"}.get(dom, dom)
+    kernel = SEARCH_KERNELS[r["search"]] if dom in ("search", "tile") else dom
     traffic = profiled_traffic(kernel, workload, n)
     if dom in ("search", "tile"):
         # arithmetic-bound: 25 binary32 operations per pair test.  The window of a
