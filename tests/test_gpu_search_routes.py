@@ -54,3 +54,96 @@ def test_documented_tile_parameters_are_the_default():
         sim = k.Simulation(k.make_config(**base, tile_threads=128), pos, vel)
         assert sim.search()[0] in (k.KMC_SEARCH_TILE, k.KMC_SEARCH_TILE_PRUNED)
         sim.close()
+
+
+def test_tile_searches_of_a_mixed_batch():
+    """Tile parameters: the plain and the pruned tile search in one launch sequence, each instance as on
+    its own with the default searches."""
+    import paper_1210_8084_gb300 as k
+    hi, cells = (1, 0.5, 0.5), (12, 6, 6)
+    ns, lams = [40_000, 30_000, 20_000], [5e-3, 1e-4, 5e-2]
+    state = [_tube(n, 200 + i, hi=hi) for i, n in enumerate(ns)]
+    insts = [dict(n=n, lam=lam, dt=1e-2, seed=300 + i) for i, (n, lam) in enumerate(zip(ns, lams))]
+    base = dict(dim_pos=3, n_cells=cells, hi=hi, bc=(WALL, PER, PER), precision=32)
+    batch = k.Simulation(k.make_config(**base, instances=insts, tile_threads=128), np.concatenate([s[0] for s in state]),
+                         np.concatenate([s[1] for s in state]))
+    assert [batch.search(i)[0] for i in range(3)] == [k.KMC_SEARCH_TILE_PRUNED, k.KMC_SEARCH_TILE, k.KMC_SEARCH_TILE_PRUNED]
+    assert batch.info().kernels_per_step == 6   # plain tile search, pruned tile search, move, scan, two scatter passes
+    batch.step(3)
+    pb, vb = batch.state()
+    off = 0
+    for i, (p, v) in enumerate(state):
+        one = k.Simulation(k.make_config(**base, lam=lams[i], dt=1e-2, seed=300 + i), p, v)
+        assert one.search()[0] in (k.KMC_SEARCH_FILTER, k.KMC_SEARCH_PAIRS, k.KMC_SEARCH_PARTICLE)
+        one.step(3)
+        po, vo = one.state()
+        assert np.array_equal(po, pb[off:off + ns[i]]) and np.array_equal(vo, vb[off:off + ns[i]]), i
+        off += ns[i]
+        one.close()
+    batch.close()
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_pruned_tile_search_at_its_own_staging_capacity(dim):
+    """tile_split alone keeps the pruned tile search's default capacity (an instance of the kernel of its own)."""
+    import paper_1210_8084_gb300 as k
+    n, cells, hi, lam, dt = (60_000, (20, 6, 6), (1, .3, .3), 1e-3, 1e-2) if dim == 3 else (200_000, (40, 40, 1), (1, 1, 1), 0.02, 5e-3)
+    bc = (WALL, PER, PER) if dim == 3 else (WALL, WALL, PER)
+    pos, vel = _tube(n, 21, hi=hi, dim=dim, bc=bc)
+    out = []
+    for split in (2, 0):
+        sim = k.Simulation(k.make_config(dim_pos=dim, n_cells=cells, hi=hi, bc=bc, lam=lam, dt=dt, seed=5, precision=32,
+                                         tile_split=split, flags=k.KMC_FLAG_RECORD), pos, vel)
+        assert sim.search()[0] == (k.KMC_SEARCH_TILE_PRUNED if split else k.KMC_SEARCH_FILTER)
+        assert sim.info().tile_cap == 1888
+        sim.step(2)
+        out.append((*sim.partners(), *sim.state()))
+        sim.close()
+    assert (out[0][0] >= 0).mean() > 0.05
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 31, 33, 64, 255, 513])
+def test_filtered_search_of_a_few_particles(n):
+    """Pruned instances are filtered at any size: part of a tile, of a group and of a warp's share."""
+    import oracle
+    import paper_1210_8084_gb300 as k
+    rng = np.random.default_rng(n)
+    cells, bc, R, dt = (6, 6, 1), (PER, WALL, PER), 0.08, 0.05
+    pos, vel = rng.random((n, 3), dtype=np.float32), rng.standard_normal((n, 3), dtype=np.float32)
+    if n <= 9:
+        pos[:, :2] = 0.4 + 0.2 * pos[:, :2]   # close enough to meet
+    pos[:, 2] = 0
+    sim = k.Simulation(k.make_config(dim_pos=2, n_cells=cells, bc=bc, sigma=np.pi * R * R, dt=dt, seed=4, precision=32,
+                                     flags=k.KMC_FLAG_RECORD), pos, vel)
+    assert sim.search()[0] == k.KMC_SEARCH_FILTER
+    sim.step(1)
+    best, _ = sim.partners()
+    sim.close()
+    P = oracle.make_params(2, cells, (0, 0, 0), (1, 1, 1), bc, R2=oracle.contact_R2(0.0, np.pi * R * R, n), dt=dt, seed=4, step=0,
+                           decide32=True)
+    assert np.array_equal(best, oracle.best_partners(P, pos.astype(np.float64), vel.astype(np.float64)))
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("n,nc,empty", [(8_003, 4, 9), (8_003, 4, 254), (400, 2, 60)])
+def test_random_partner_variant_is_the_same_by_thread_warp_and_block(n, nc, empty, prec):
+    """The launch gives a cell a thread, a warp or a block by the mean number of particles; empty instances beside
+    the same one lower the mean.  Bit for bit, over cells in which nearly all candidates depend on others."""
+    import paper_1210_8084_gb300 as k
+    dtype = np.float32 if prec == 32 else np.float64
+    pos, vel = _tube(n, 30, dtype)
+    base = dict(dim_pos=3, n_cells=(nc, 1, 1), bc=(WALL, PER, PER), precision=prec, flags=k.KMC_FLAG_DSMC)
+    one = dict(n=n, lam=1e-3, dt=2e-2, seed=77)
+    out = []
+    for extra in (0, empty):
+        insts = [one] + [dict(n=0, lam=1e-3, dt=2e-2, seed=i) for i in range(extra)]
+        cfg = k.make_config(**base, instances=insts) if extra else k.make_config(**base, lam=1e-3, dt=2e-2, seed=77)
+        sim = k.Simulation(cfg, pos, vel)
+        sim.step(3)
+        out.append(sim.state())
+        sim.close()
+    assert not np.array_equal(out[0][1], vel)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
