@@ -300,13 +300,10 @@ inline bool filter_fits(const InstDev& I, const Geo& g, double dt) {
 #else
 #define KMC_HOST_DEVICE
 #endif
-// Pieces of `size` positions that positions [q0, q1) touch (counted from position 0) and
-// that they fill (counted from q0).  Positions go up to 2^31 - 2: nothing is rounded up past them.
+// Pieces of `size` positions, counted from position 0, that positions [q0, q1) touch.
+// Positions go up to 2^31 - 2: nothing is rounded up past them.
 KMC_HOST_DEVICE inline int32_t pieces_touched(int32_t q0, int32_t q1, int32_t size) {
     return q1 > q0 ? (q1 - 1) / size - q0 / size + 1 : 0;
-}
-KMC_HOST_DEVICE inline int32_t pieces_filled(int32_t q0, int32_t q1, int32_t size) {
-    return q1 > q0 ? (q1 - q0 - 1) / size + 1 : 0;
 }
 
 // Particles the buffers of a state of n hold: whole groups of 32, so that the filtered

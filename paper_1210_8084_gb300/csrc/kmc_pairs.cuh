@@ -136,10 +136,11 @@ __global__ void __launch_bounds__(32, kPairsBlocks) pairs_search_kernel(Bufs<flo
                                      DIM == 3 ? (float)(1 - (int)(cd >> 2 & 3u)) * G.L[1] : (float)(1 - (int)(cd >> 4 & 3u)) * G.L[1],
                                      DIM == 3 ? (float)(1 - (int)(cd >> 4 & 3u)) * G.L[2] : 0.f};
                 const bool shifted = sh[0] != 0.f || sh[1] != 0.f || sh[2] != 0.f;
-                const int32_t chunks = pieces_filled(a0, a1, kPairsChunk);
-                for (int32_t chunk = 0; chunk < chunks; ++chunk) {
-                    const int32_t base = a0 + chunk * kPairsChunk;
-                    const int n = min(kPairsChunk, a1 - base);
+                // counted down: positions go up to 2^31 - 2, and a step past a1 could pass 2^31
+                uint32_t next = (uint32_t)a0;
+                for (int32_t left = a1 - a0; left > 0; left -= kPairsChunk, next += kPairsChunk) {
+                    const int32_t base = (int32_t)next;
+                    const int n = min(kPairsChunk, left);
                     __syncwarp();
                     // a pair farther than both of its particles' closest so far is no pair
                     // (a stale value is a larger one): negated bounds on its distance^2
