@@ -278,9 +278,12 @@ __device__ __forceinline__ double unfix(unsigned long long a, int e) {
     return x == 0.0 ? 0.0 : __longlong_as_double(__double_as_longlong(x) - ((long long)e << 52));
 }
 
-// a / b from the correctly rounded reciprocal r of b: one Newton step on the
-// quotient, correctly rounded by Markstein's theorem (IBM J. Res. Dev. 34, 1990)
-// for operands away from the ends of the range, as here.
+// a / b, correctly rounded, from the correctly rounded reciprocal r of an integer b
+// below 2^32 (a count, or 3), for quotients away from the ends of the range, as here.
+// a r is within 2^-52 of the quotient, the step on its residual then within 2^-104 before
+// the last rounding.  That rounds as the quotient does, because no quotient comes as near
+// to the middle m of two neighbours: |a - b m| is not zero (a would need 54 bits) and a multiple
+// of m's last place, 2^-54 m or more, so |a / b - m| is at least 2^-86 m.
 __device__ __forceinline__ double div_rcp(double a, double b, double r) {
     const double q = a * r;
     return fma(fma(-q, b, a), r, q);
