@@ -30,10 +30,10 @@
 // below 2^-17 D^2 with D the reach R + 2 v_max dt) and by that of the product's
 // sum (16 terms of 12 X^2 in all: 2^-18 of it).  kmc_scan.cu holds the constants.
 //
-// Bound by instruction issue (71 % of the slots, 10,400 instructions per 32 homes of the
+// Bound by instruction issue (71 % of the slots, 9,900 instructions per 32 homes of the
 // 16M tube).  The searches it replaced -> this one, GB300, ms per step: 3-D Sod tube,
 // 512M particles 423 -> 191, 16M 14.6 -> 6.3, 21M at 20 per c-bin 25.0 -> 3.6; Sedov
-// blast, 8M 15.3 -> 1.14; binary64 slab tube, 200k 2.33 -> 0.27.  Per 32 homes of the 16M
+// blast, 8M 15.3 -> 1.14; binary64 slab tube, 200k 2.33 -> 0.26.  Per 32 homes of the 16M
 // tube: 431 tiles of 8 candidates in the window, 135 past the box check, 411 pairs
 // past the filter.
 #pragma once

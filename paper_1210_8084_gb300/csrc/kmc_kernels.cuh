@@ -2629,7 +2629,7 @@ __device__ __forceinline__ uint32_t tags_below(const uint32_t* __restrict__ t, u
 // a narrow range), the buckets divide the cell's own range, and the tags are placed
 // themselves, to be compared four per load where a few far ids still crowd the
 // others.  Both scatter passes with this kernel, GB300, ms: 64M particles in 262,144 cells
-// (quadrants) 5.16 -> 2.36; 4M in 2000 cells 0.94 -> 0.11, with ids in cell order 0.94 ->
+// (quadrants) 5.16 -> 2.15; 4M in 2000 cells 0.94 -> 0.11, with ids in cell order 0.94 ->
 // 0.12 (1.39 with the instance's range alone), the same but four far ids per cell 0.63.
 template <typename T, int CAP, int TPB>
 __global__ void __launch_bounds__(TPB) rank_cells_kernel(Bufs<T> b, uint32_t above) {
@@ -2910,8 +2910,10 @@ __global__ void __launch_bounds__(kThreads) dsmc_kernel(Bufs<T> b) {
 // rate), the accepted ones are gathered so that full warps take the binary64
 // collision.  The order of dependent candidates, and so every bit, is that of the
 // sequence.  4M particles in 2000 cells, GB300: 26.6 ms with one thread per cell (a
-// chain of dependent loads and binary64 operations per candidate) -> 0.95 ms,
-// bound by the binary64 collisions and the rounds' barriers.
+// chain of dependent loads and binary64 operations per candidate) -> 0.95 ms.  Of
+// 400 such cells (800k particles, one wave of blocks) the rounds' barriers take 22 of 38
+// cycles between a warp's issues, as a batch's last dependent candidates wait for one
+// another; the binary64 pipe is 46 % busy on average, 74 % on the busiest SM.
 template <int TPC>
 __device__ __forceinline__ void dsmc_sync() {
     if (TPC == 32) __syncwarp();
