@@ -512,7 +512,8 @@ __device__ __forceinline__ bool poca_test_sh(const GeoT<T>& G, const T xi[3], co
 }
 
 // Search window of one dimension in search-cell coordinates: within k cells of
-// g and inside the c-bins c-1 .. c+1; cut at walls.  A periodic window is kept
+// g and inside the c-bins c-1 .. c+1; cut at walls.  Of three periodic c-bins every
+// one is a neighbour, the one across also on the near side (c + 2 or c - 2): no cut there.  A periodic window is kept
 // unwrapped (t in (-M, 2M); image shift +L below 0, -L above M-1).  When every
 // cell of the window lies less than half a box (minus half a cell) from the
 // particle's cell, all candidates of a row share one image and the shift is
@@ -524,8 +525,9 @@ struct Win {
 };
 __device__ __forceinline__ Win window_1d(int g, int c, int s, int M, int k, bool wall) {
     Win w;
-    w.lo = max(g - k, (c - 1) * s);
-    w.hi = min(g + k, (c + 2) * s - 1);
+    const bool cut = wall || M != 3 * s;
+    w.lo = cut ? max(g - k, (c - 1) * s) : g - k;
+    w.hi = cut ? min(g + k, (c + 2) * s - 1) : g + k;
     w.amb = false;
     if (wall) {
         w.lo = max(w.lo, 0);
