@@ -367,6 +367,28 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
     }
 }
 
+// Frame blocks that a warp of the filtered search walks, over all its runs of homes: the
+// frames as the step's constants set them (kmc_scan.cu, filter_constants), n_row homes
+// per row of search cells, spread over its length.
+double walk_blocks(const kmc_handle* h, const InstDev& I, bool chi, double s, double n_row) {
+    const int F = h->dim - 1;
+    const double R = sqrt(I.R2), D = R + 2.0 * s, Re = I.sym ? R : 0.125 * R;
+    double reach = 0.0;
+    for (int d = 0; d <= F; ++d) reach = std::max(reach, std::min(D, 2.0 * I.s[d] * I.w[d]));
+    const double width = 2.0 * ((chi ? std::min(200.0 * R, 400.0 * s) : 46.0 * sqrt(Re * Re + s * s / 16.0)) - reach - s);
+    const double rows = std::max(n_row, 1e-3);
+    double blocks = 1.0 + 32.0 / rows;   // runs
+    for (int d = 0; d <= F; ++d) {
+        int sh = 0;
+        while ((1 << sh) < I.M[d] && (double)std::min(2 << sh, I.M[d]) * I.w[d] <= width) ++sh;
+        const double k = ceil((1.001 * D + 1e-5 * h->geo.L[d]) / I.w[d]), M = (double)I.M[d];
+        double cells = std::min(2.0 * k + 1.0, (double)std::min(3 * I.s[d], I.M[d]));
+        if (d == F) cells = std::min(cells + std::min(1.0, 32.0 / rows) * M, M + 1.0);
+        blocks *= 1.0 + (cells - 1.0) / std::min((double)(1 << sh), M);
+    }
+    return blocks;
+}
+
 // Costs of an instance's searches where no option asks for a particular one, and the
 // forms of the filtered and the pair search.  Estimates per particle: `occ` is the particles' mean occupancy of their c-bin; `cand`
 // the candidates of the first step's window, `within` those inside the contact
@@ -378,7 +400,8 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
 // falls to its closest candidate: twice the pairs, but few of them left (a tenth
 // at 150-270 particles per c-bin of the quadrant workload).  Binary64 (its exact test runs at 1/64 of the
 // binary32 rate) filters by criterion 1 too, unless a window holds few candidates.
-SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms, double occ) {
+// `c_rows`: rows of c-bins (along the last dimension) that hold particles.
+SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms, double occ, double c_rows) {
     const double dt0 = (I.adaptive && vmax > 0.0) ? I.dx_min / vmax : I.dt;
     const double R = sqrt(I.R2), reach = 1.001 * (R + 2.0 * vmax * dt0), rho = sqrt(I.R2 + 1.2 * vrms * vrms * dt0 * dt0);
     double cand = occ, within = occ, near = occ;
@@ -397,8 +420,9 @@ SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms,
         h->filter_chi = 1;   // criterion 1 leaves about the passing ones
         hits = std::min(hits, 4.0 * passing);
     }
-    double rows = 1.0, n_row = occ * h->geo.n[h->dim - 1];
+    double rows = 1.0, n_row = occ * h->geo.n[h->dim - 1], s_rows = c_rows;
     for (int d = 0; d + 1 < h->dim; ++d) {
+        s_rows *= I.s[d];
         const double k = ceil((reach + 1e-5 * h->geo.L[d]) / I.w[d]);
         rows *= std::min(2.0 * k + 1.0, (double)std::min(3 * I.s[d], I.M[d]));
         n_row /= I.s[d];
@@ -406,13 +430,16 @@ SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms,
     I.close = passing > kPairsClose ? 1 : 0;
     if (h->precision == 64) {
         h->filter_chi = 1;
-        SearchCosts c = search_costs64((double)h->n, cand, n_row);
+        const double mean_row = (double)I.n / std::max(s_rows, 1.0);
+        SearchCosts c = search_costs64(h->dim, (double)h->n, cand, n_row, 1.0 + 32.0 / std::max(mean_row, 1e-3),
+                                       walk_blocks(h, I, true, vmax * dt0, mean_row));
         if (!filter_fits(I, h->geo, dt0)) c.ps[kSearchFilter] = INFINITY;
         return c;
     }
     bool wraps = false;   // with room for v_max to grow (InstDyn::p_image)
     for (int d = 0; d < h->dim; ++d) wraps = wraps || (h->geo.bc[d] == KMC_BC_PERIODIC && reach > 0.4 * h->geo.L[d]);
-    return search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, wraps, (double)h->n, cand, hits, passing, rows, n_row);
+    const double walks = walk_blocks(h, I, h->filter_chi != 0, vmax * dt0, (double)I.n / std::max(s_rows, 1.0));
+    return search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, wraps, (double)h->n, cand, hits, passing, rows, n_row, walks);
 }
 
 // The searches of a handle's instances: pruned ones are filtered, the others take the
@@ -821,16 +848,24 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         if (!okc) return bail(fail(h, KMC_ECUDA, "search-grid statistics failed"));
         uint64_t keys = 0;
         std::vector<uint32_t> max_occ(h->n_inst, 0u);
-        std::vector<double> vmax(h->n_inst, 0.0), occ(h->n_inst, 0.0);
+        std::vector<double> vmax(h->n_inst, 0.0), occ(h->n_inst, 0.0), c_rows(h->n_inst, 0.0);
+        const int64_t row_bins = h->bins_per_inst / h->geo.n[h->dim - 1];   // c-bin = row + rows * c of the last dimension
+        std::vector<char> held((size_t)row_bins);
         std::vector<SearchCosts> costs;
         for (int i = 0; i < h->n_inst; ++i) {
             uint32_t mx = 0;
             uint64_t sq = 0;   // of the occupancies
             const uint32_t* hist_i = hist_h.data() + (size_t)(i * h->bins_per_inst);
-            for (int64_t b = 0; b < h->bins_per_inst; ++b) {
-                mx = std::max(mx, hist_i[b]);
-                sq += (uint64_t)hist_i[b] * hist_i[b];
+            std::fill(held.begin(), held.end(), 0);
+            for (int64_t z = 0; z < h->bins_per_inst; z += row_bins) {
+                for (int64_t r = 0; r < row_bins; ++r) {
+                    const uint32_t c = hist_i[z + r];
+                    mx = std::max(mx, c);
+                    sq += (uint64_t)c * c;
+                    held[(size_t)r] |= c > 0;
+                }
             }
+            c_rows[i] = (double)std::count(held.begin(), held.end(), 1);
             max_occ[i] = mx;
             double v2;
             memcpy(&v2, &vm_h[i], sizeof(double));
@@ -845,7 +880,8 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
         for (int i = 0; i < h->n_inst; ++i) {
             double sample[2];
             memcpy(sample, &vm_h[(size_t)h->n_inst + 2 * i], sizeof(sample));
-            costs.push_back(estimate_search(h, h->inst_h[i], vmax[i], sample[1] > 0.0 ? sqrt(sample[0] / sample[1]) : 0.0, occ[i]));
+            costs.push_back(estimate_search(h, h->inst_h[i], vmax[i], sample[1] > 0.0 ? sqrt(sample[0] / sample[1]) : 0.0, occ[i],
+                                            c_rows[i]));
         }
         choose_searches(h, costs);
         for (auto& I : h->inst_h) {

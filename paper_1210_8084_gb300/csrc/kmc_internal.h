@@ -354,34 +354,46 @@ inline int rank_launches(int64_t n, uint32_t n_keys) {
 // window that may reach around a periodic box (`wraps`) makes the pair search decide
 // every pair exactly (4,900 particles, 440 candidates: 138 us, 113, 1240).
 // A warp's homes test the union of their windows, 32 particles more per row, and a
-// warp whose homes lie in several rows walks once per row (`runs`).
+// warp whose homes lie in several rows walks once per row (`runs`).  `walks`: frame blocks
+// that a warp of the filtered search visits in all (walk_blocks); up to ten are in the fit
+// above.  Particles spread thinly beside a dense cluster, with contact distance and
+// displacement far below a cell, make hundreds: 2.1M particles, 260 candidates 19.0 ms filtered,
+// 0.67 one thread per particle (without this term the filter was chosen).
 struct SearchCosts {
     double ps[3];   // kSearchDirect, kSearchFilter, kSearchPairs
 };
+inline double walk_cost(double walks, double n_all) { return walks > 10.0 ? (10.0 + 1.5e6 / n_all) * (walks - 10.0) : 0.0; }
 inline SearchCosts search_costs(int dim, bool split, bool wraps, double n_all, double cand, double hits, double passing,
-                                double rows, double n_row) {
+                                double rows, double n_row, double walks) {
     const double tests = cand + 32.0 * rows, runs = 1.0 + 32.0 / (n_row > 1.0 ? n_row : 1.0);
     SearchCosts c;
     c.ps[kSearchDirect] = dim == 2 ? 25.0 + 0.85 * cand : split ? 70.0 + 1.3 * cand : 45.0 + 0.85 * cand;
     c.ps[kSearchFilter] = (130.0 + 0.07 * cand + 6.0 * hits) * runs;
     c.ps[kSearchPairs] = (dim == 3 ? 38.0 + 0.30 * tests : 24.0 + 0.28 * tests) * runs + 3.0 * (passing < 64.0 ? passing : 64.0);
     c.ps[kSearchDirect] += (20.0 + 0.27 * cand) * 1e6 / n_all;
-    c.ps[kSearchFilter] += (45.0 + 10.0 * runs + 0.3 * hits) * 1e6 / n_all;
+    c.ps[kSearchFilter] += (45.0 + 10.0 * runs + 0.3 * hits) * 1e6 / n_all + walk_cost(walks, n_all);
     c.ps[kSearchPairs] += (35.0 + 0.04 * cand) * 1e6 / n_all;
     if (wraps) c.ps[kSearchPairs] *= 20.0;
     return c;
 }
 // Binary64: one thread per particle or filtered, per particle of a handle of n_all.  Up to
-// some 80,000 particles a search is one wave, its time that of a particle's walk or of a
-// group's runs.  us per search, measured / estimated, one thread per particle and filtered
-// (slab tubes): 30,000 particles, 10 candidates, 13 per row of cells 89 / 122, 236 / 284;
-// 11,000, 112, 21 per row 380 / 505, 328 / 198; 97,000, 43, 21 per row 554 / 490, 247 / 267;
-// 1M, 11, 33 per row 1190 / 1270, 940 / 950; 1M, 67, 65 per row 4600 / 4800, 1000 / 910.
-inline SearchCosts search_costs64(double n_all, double cand, double n_row) {
-    const double runs = 1.0 + 32.0 / (n_row > 1.0 ? n_row : 1.0);
+// some 100,000 particles a search is about one wave, its time that of a particle's walk or
+// of a group's runs and frame blocks; fitted to 410 states of 2,000-100,000 particles.  us per
+// search, measured / estimated, one thread per particle and filtered: 2-D, 20,000 particles, 13
+// candidates, 3 blocks 30 / 41, 85 / 65; 3-D, 5,600, 55, 8 blocks 95 / 112, 110 / 104; above, slab
+// tubes: 1M, 11, 33 per row 1190 / 1270, 940 / 950; 1M, 67, 65 per row 4600 / 4800, 1000 / 910.
+// `runs` here is the mean over the particles (few per row count fully).
+inline SearchCosts search_costs64(int dim, double n_all, double cand, double n_row, double runs, double walks) {
+    const double L = 1e6 / n_all;
     SearchCosts c;
-    c.ps[kSearchDirect] = (45.0 + 3.4 * cand) * 1e6 / n_all + 500.0 + 60.0 * cand;
-    c.ps[kSearchFilter] = 75.0 * runs * 1e6 / n_all + 800.0;
+    if (n_all < 1e5) {
+        c.ps[kSearchDirect] = dim == 3 ? (55.0 + 0.9 * cand) * L + 80.0 + 24.0 * cand : (20.0 + 0.84 * cand) * L + 20.0 + 24.0 * cand;
+        c.ps[kSearchFilter] = dim == 3 ? (76.0 + 3.0 * runs + 1.9 * walks) * L + 360.0 + 66.0 * walks
+                                       : (40.0 + 3.0 * walks) * L + 320.0 * runs + 4.4 * cand;
+    } else {
+        c.ps[kSearchDirect] = (45.0 + 3.4 * cand) * L + 500.0 + 60.0 * cand;
+        c.ps[kSearchFilter] = 75.0 * (1.0 + 32.0 / (n_row > 1.0 ? n_row : 1.0)) * L + 800.0 + walk_cost(walks, n_all);
+    }
     c.ps[kSearchPairs] = c.ps[kSearchDirect] + c.ps[kSearchFilter];   // binary32 only
     return c;
 }

@@ -144,10 +144,10 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     const double n_row = (double)n / n_rows;
     I.search = n == 0 ? kSearchDirect
                : sizeof(T) == 8
-                   ? cheapest_search(search_costs64((double)n, cand, n_row),
+                   ? cheapest_search(search_costs64(g.dim, (double)n, cand, n_row, 1.0 + 32.0 / fmax(n_row, 1.0), 8.0),
                                      1u << kSearchDirect | (filter_fits(I, g, I.dt) ? 1u << kSearchFilter : 0u))
                    : cheapest_search(search_costs(g.dim, split, wraps, (double)n, cand, I.sym ? 0.25 * near : 0.1 * cand, passing,
-                                                    rows, n_row), 7u);
+                                                    rows, n_row, 0.0), 7u);
     I.close = passing > kPairsClose ? 1 : 0;
     I.chi = sizeof(T) == 8 ? 1 : 0;
     filter_lengths(I, g, sizeof(T) == 8);

@@ -147,3 +147,25 @@ def test_random_partner_variant_is_the_same_by_thread_warp_and_block(n, nc, empt
     assert not np.array_equal(out[0][1], vel)
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec,n,cells", [(32, 400_000, (60, 16, 16)), (32, 2_000_000, (120, 32, 32)), (64, 436_649, (109, 19, 19))])
+def test_thin_particles_beside_a_cluster(prec, n, cells):
+    """A third of the particles in a hundredth of the box, contact distance and displacement far below a cell: the
+    filtered search would walk hundreds of frame blocks for the thin rows (24 times as long as one thread per particle)."""
+    import paper_1210_8084_gb300 as k
+    rng = np.random.default_rng(3)
+    dtype = np.float32 if prec == 32 else np.float64
+    hi = np.array([1.0, cells[1] / cells[0], cells[2] / cells[0]])
+    pos = rng.random((n, 3)) * 0.9999
+    pos[:n // 3] = 0.4 + 0.1 * pos[:n // 3]
+    pos, vel = (pos * hi).astype(dtype), rng.standard_normal((n, 3)).astype(dtype)
+    R = (0.013 if prec == 32 else 0.004) / cells[0]
+    ms = []
+    for flags in (0, k.KMC_FLAG_NO_TILE_SEARCH):
+        sim = k.Simulation(k.make_config(dim_pos=3, n_cells=cells, hi=tuple(hi), bc=(PER, PER, WALL), sigma=np.pi * R * R,
+                                         dt=0.011 / cells[0], seed=1, precision=prec, flags=flags), pos, vel)
+        sim.step(1)
+        ms.append(min(sim.step_profiled(1)["search"] for _ in range(4)))
+        sim.close()
+    assert ms[0] < 1.5 * ms[1], ms
