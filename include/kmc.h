@@ -67,8 +67,8 @@ extern "C" {
 #define KMC_FLAG_RECORD 1   /* keep each particle's closest candidate and partner of the last step */
 #define KMC_FLAG_NO_GRAPH 2 /* launch kernels directly instead of replaying a captured CUDA graph (by default
                              * kmc_step launches one graph that loops over all its steps on the device) */
-/* The search of an instance (one particle per thread, filtered by tensor-core products, or a lane per particle
- * against staged pairs) is chosen by its estimated cost.  The next two flags, KMC_FLAG_NO_TILE_PRUNE and the tile
+/* The search of an instance (one particle per thread, filtered by tensor-core products, a lane per particle
+ * against staged pairs or, small single runs, one block per c-bin) is chosen by its estimated cost.  The next two flags, KMC_FLAG_NO_TILE_PRUNE and the tile
  * parameters of kmc_config ask for one of the other searches instead; speed only, never results. */
 #define KMC_FLAG_STAGED_SEARCH 4 /* stage tile neighbourhoods in shared memory (3-D; same results as the direct search) */
 #define KMC_FLAG_NO_TILE_SEARCH 8 /* one particle per thread for every instance (same results) */
@@ -210,7 +210,7 @@ KMC_API int kmc_step(kmc_handle* h, int nsteps, int want_moments);
 
 /* Phases of one step, in launch order, for kmc_step_profiled. */
 #define KMC_PHASE_SEARCH 0   /* closest candidate per particle (criteria 1-3) */
-#define KMC_PHASE_TILE 1     /* the same, one block per c-bin, where a flag or tile parameters ask for it */
+#define KMC_PHASE_TILE 1     /* the same, one block per c-bin: small single runs, or where a flag or tile parameters ask for it */
 #define KMC_PHASE_MOVE 2     /* pairs, scattering, free flight, walls, next key and histogram */
 #define KMC_PHASE_SCAN 3     /* exclusive scan of the key histogram */
 #define KMC_PHASE_SCATTER 4  /* counting-sort scatter into (key, id) order */

@@ -438,12 +438,33 @@ SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms,
     }
     bool wraps = false;   // with room for v_max to grow (InstDyn::p_image)
     for (int d = 0; d < h->dim; ++d) wraps = wraps || (h->geo.bc[d] == KMC_BC_PERIODIC && reach > 0.4 * h->geo.L[d]);
-    const double walks = walk_blocks(h, I, h->filter_chi != 0, vmax * dt0, (double)I.n / std::max(s_rows, 1.0));
-    return search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, wraps, (double)h->n, cand, hits, passing, rows, n_row, walks);
+    const double mean_row = (double)I.n / std::max(s_rows, 1.0);
+    const double walks = walk_blocks(h, I, h->filter_chi != 0, vmax * dt0, mean_row);
+    SearchCosts c = search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, wraps, (double)h->n, cand, hits, passing, rows,
+                                 n_row, walks);
+    // Small single runs where a block per c-bin takes less (us, fitted to 320 pruned states of up
+    // to 130,000 particles and 190 plain ones of up to 20,000; a run's latency decides): the
+    // filtered search was up to 4.9 times as long (4,254 particles in 1,044 c-bins, both
+    // scatter passes included, 74 us; tile 41).  The others pay for their blocks over all c-bins alike.
+    const double n = (double)I.n, bins = (double)h->bins_per_inst;
+    const bool three = h->dim == 3;
+    if (h->n_inst == 1 && I.prune && I.n < 130000) {
+        const double filter = 20.0 + 2.6 * walks + (350.0 + 25.0 * walks + 3.0 * hits) * 1e-6 * n;
+        const double tile = three ? 13.0 + 0.0146 * bins + (0.016 + 4.4e-7 * n) * cand : 7.0 + 0.009 * bins + (0.048 + 5.8e-7 * n) * cand;
+        c.tile = tile < filter;
+    } else if (h->n_inst == 1 && I.s[0] == 1 && I.s[1] == 1 && I.s[2] == 1 && I.n < 20000) {
+        const double runs = 1.0 + 32.0 / std::max(n_row, 1.0);
+        const double filter = std::max(three ? 40.0 + 0.09 * hits + 400e-6 * n : 28.0 + 0.117 * hits + 145e-6 * n * walks,
+                                       45.0 + 10.0 * runs + 0.3 * hits);
+        const int k = cheapest_search(c, 7u);
+        const double tile = 5.0 + (three ? 0.008 * bins + (0.162 + 1.2e-7 * n) * cand : 0.0077 * bins + (0.13 + 4.7e-7 * n) * cand);
+        c.tile = tile < (k == kSearchFilter ? filter : c.ps[k] * 1e-6 * n);
+    }
+    return c;
 }
 
-// The searches of a handle's instances: pruned ones are filtered, the others take the
-// set of searches that costs least.  A further search reads every
+// The searches of a handle's instances: pruned ones are filtered (small single runs: or
+// tiled), the others take the set of searches that costs least.  A further search reads every
 // particle once more (6 ps each: a 158M-particle ensemble took 30.0 ms with the three
 // cheapest per instance and 27.9 ms with one).  A handle with pruned instances uses
 // no pair search.
@@ -475,7 +496,7 @@ void choose_searches(kmc_handle* h, const std::vector<SearchCosts>& cost) {
     }
     for (int i = 0; i < h->n_inst; ++i) {
         InstDev& I = h->inst_h[i];
-        I.search = I.n == 0 ? kSearchDirect : I.prune ? kSearchFilter : cheapest_search(cost[i], best);
+        I.search = I.n == 0 ? kSearchDirect : cost[i].tile ? kSearchTile : I.prune ? kSearchFilter : cheapest_search(cost[i], best);
     }
 }
 
@@ -918,8 +939,15 @@ int kmc_init(const kmc_config* cfg, int64_t n, const void* pos, const void* vel,
                 continue;
             }
             if (choose) {
-                I.tiled = 0;
+                I.tiled = I.search == kSearchTile;
                 I.prune = I.prune && I.n > 0;
+                if (I.tiled) {
+                    I.search = kSearchDirect;
+                    h->any_tiled = 1;
+                    h->any_plain_tiled |= !I.prune;
+                    prune_any |= I.prune;
+                    continue;
+                }
                 h->filtered |= I.search == kSearchFilter;
                 if (I.search == kSearchPairs) (I.close ? close : open) += I.n;
                 h->any_direct |= I.n > 0 && I.search == kSearchDirect;

@@ -41,6 +41,7 @@ constexpr unsigned long long kNoPartner = ~0ull;  // partner key of a particle w
 constexpr int kSearchDirect = 0;       // one thread per particle
 constexpr int kSearchFilter = 1;       // kmc_filter.cuh
 constexpr int kSearchPairs = 2;        // kmc_pairs.cuh, binary32
+constexpr int kSearchTile = 3;         // tile search, pruned on half c-bins (small single runs; InstDev::tiled)
 constexpr int kMomItems = 4;           // moments: consecutive particles per thread
 constexpr int kStageThreads = 256;     // staged search: threads per tile
 
@@ -360,7 +361,8 @@ inline int rank_launches(int64_t n, uint32_t n_keys) {
 // displacement far below a cell, make hundreds: 2.1M particles, 260 candidates 19.0 ms filtered,
 // 0.67 one thread per particle (without this term the filter was chosen).
 struct SearchCosts {
-    double ps[3];   // kSearchDirect, kSearchFilter, kSearchPairs
+    double ps[3];           // kSearchDirect, kSearchFilter, kSearchPairs
+    bool tile = false;      // a small single run whose tile search costs less than any of them
 };
 inline double walk_cost(double walks, double n_all) { return walks > 10.0 ? (10.0 + 1.5e6 / n_all) * (walks - 10.0) : 0.0; }
 inline SearchCosts search_costs(int dim, bool split, bool wraps, double n_all, double cand, double hits, double passing,

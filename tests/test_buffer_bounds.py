@@ -26,8 +26,9 @@ for prec in (32, 64):
     dtype = np.float32 if prec == 32 else np.float64
     for n in list(range(0, 42)) + [255, 1001]:
         pos, vel = np.full((n, 3), 0.5, dtype), np.zeros((n, 3), dtype)
-        # a contact distance just under half a c-bin: a binary32 handle takes the filtered search
-        cfg = k.make_config(dim_pos=2, n_cells=(6, 6, 1), sigma=math.pi * (0.48 / 6) ** 2, dt=1e-3, precision=prec,
+        # a contact distance just under half a c-bin: a binary32 batch takes the filtered search
+        one = dict(sigma=math.pi * (0.48 / 6) ** 2, lam=1.0, dt=1e-3)
+        cfg = k.make_config(dim_pos=2, n_cells=(6, 6, 1), instances=[dict(one, n=n), dict(one, n=0)], precision=prec,
                             flags=k.KMC_FLAG_NO_GRAPH)
         h = ctypes.c_void_p()
         ptr = lambda a: a.ctypes.data_as(ctypes.c_void_p)

@@ -106,7 +106,7 @@ def test_pruned_tile_search_at_its_own_staging_capacity(dim):
 
 @pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 31, 33, 64, 255, 513])
 def test_filtered_search_of_a_few_particles(n):
-    """Pruned instances are filtered at any size: part of a tile, of a group and of a warp's share."""
+    """Pruned instances of a batch are filtered at any size: part of a tile, of a group and of a warp's share."""
     import oracle
     import paper_1210_8084_gb300 as k
     rng = np.random.default_rng(n)
@@ -115,9 +115,10 @@ def test_filtered_search_of_a_few_particles(n):
     if n <= 9:
         pos[:, :2] = 0.4 + 0.2 * pos[:, :2]   # close enough to meet
     pos[:, 2] = 0
-    sim = k.Simulation(k.make_config(dim_pos=2, n_cells=cells, bc=bc, sigma=np.pi * R * R, dt=dt, seed=4, precision=32,
-                                     flags=k.KMC_FLAG_RECORD), pos, vel)
-    assert sim.search()[0] == k.KMC_SEARCH_FILTER
+    insts = [dict(n=m, sigma=np.pi * R * R, lam=1.0, dt=dt, seed=4) for m in (n, 0)]
+    sim = k.Simulation(k.make_config(dim_pos=2, n_cells=cells, bc=bc, instances=insts, precision=32, flags=k.KMC_FLAG_RECORD),
+                       pos, vel)
+    assert sim.search(0)[0] == k.KMC_SEARCH_FILTER
     sim.step(1)
     best, _ = sim.partners()
     sim.close()
@@ -169,3 +170,23 @@ def test_thin_particles_beside_a_cluster(prec, n, cells):
         ms.append(min(sim.step_profiled(1)["search"] for _ in range(4)))
         sim.close()
     assert ms[0] < 1.5 * ms[1], ms
+
+
+@pytest.mark.parametrize("n,dim,cells,hi,R,dt,search", [
+    (3_708, 3, (39, 6, 6), (1, 6 / 39, 6 / 39), 0.49, 0.11, 4), (10_860, 2, (85, 8, 1), (1, 8 / 85, 1), 0.022, 0.3, 4),
+    (4_254, 3, (29, 6, 6), (1, 6 / 29, 6 / 29), 0.022, 0.13, 4), (2_189, 3, (34, 4, 4), (1, 4 / 34, 4 / 34), 0.03, 0.34, 3)])
+def test_small_runs_take_no_longer_than_a_block_per_c_bin(n, dim, cells, hi, R, dt, search):
+    """A few thousand particles in hundreds of c-bins: the tile searches' latency beats the filter's (up to 4.9 times)."""
+    import paper_1210_8084_gb300 as k
+    bc = (PER, PER, WALL)
+    pos, vel = _tube(n, 41, hi=hi, dim=dim, bc=bc)
+    pos[:, 0] = np.minimum(pos[:, 0], np.nextafter(np.float32(1), np.float32(0)))
+    base = dict(dim_pos=dim, n_cells=cells, hi=hi, bc=bc, sigma=np.pi * (R / cells[0]) ** 2, dt=dt / cells[0], seed=1, precision=32)
+    ms = []
+    for tile in (0, 1534):   # not the default capacity: asks for the tile search
+        sim = k.Simulation(k.make_config(**base, tile_cap=tile), pos, vel)
+        assert sim.search()[0] == search
+        sim.step(1)
+        ms.append(min(p["search"] + p["tile"] for p in (sim.step_profiled(1) for _ in range(6))))
+        sim.close()
+    assert ms[0] < 1.3 * ms[1], ms
