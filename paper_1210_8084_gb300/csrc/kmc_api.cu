@@ -367,28 +367,6 @@ void choose_subdivision(const kmc_handle* h, InstDev& I, double vmax, uint32_t m
     }
 }
 
-// Frame blocks that a warp of the filtered search walks, over all its runs of homes: the
-// frames as the step's constants set them (kmc_scan.cu, filter_constants), n_row homes
-// per row of search cells, spread over its length.
-double walk_blocks(const kmc_handle* h, const InstDev& I, bool chi, double s, double n_row) {
-    const int F = h->dim - 1;
-    const double R = sqrt(I.R2), D = R + 2.0 * s, Re = I.sym ? R : 0.125 * R;
-    double reach = 0.0;
-    for (int d = 0; d <= F; ++d) reach = std::max(reach, std::min(D, 2.0 * I.s[d] * I.w[d]));
-    const double width = 2.0 * ((chi ? std::min(200.0 * R, 400.0 * s) : 46.0 * sqrt(Re * Re + s * s / 16.0)) - reach - s);
-    const double rows = std::max(n_row, 1e-3);
-    double blocks = 1.0 + 32.0 / rows;   // runs
-    for (int d = 0; d <= F; ++d) {
-        int sh = 0;
-        while ((1 << sh) < I.M[d] && (double)std::min(2 << sh, I.M[d]) * I.w[d] <= width) ++sh;
-        const double k = ceil((1.001 * D + 1e-5 * h->geo.L[d]) / I.w[d]), M = (double)I.M[d];
-        double cells = std::min(2.0 * k + 1.0, (double)std::min(3 * I.s[d], I.M[d]));
-        if (d == F) cells = std::min(cells + std::min(1.0, 32.0 / rows) * M, M + 1.0);
-        blocks *= 1.0 + (cells - 1.0) / std::min((double)(1 << sh), M);
-    }
-    return blocks;
-}
-
 // Costs of an instance's searches where no option asks for a particular one, and the
 // forms of the filtered and the pair search.  Estimates per particle: `occ` is the particles' mean occupancy of their c-bin; `cand`
 // the candidates of the first step's window, `within` those inside the contact
@@ -432,14 +410,14 @@ SearchCosts estimate_search(kmc_handle* h, InstDev& I, double vmax, double vrms,
         h->filter_chi = 1;
         const double mean_row = (double)I.n / std::max(s_rows, 1.0);
         SearchCosts c = search_costs64(h->dim, (double)h->n, cand, n_row, 1.0 + 32.0 / std::max(mean_row, 1e-3),
-                                       walk_blocks(h, I, true, vmax * dt0, mean_row));
+                                       walk_blocks(I, h->geo, true, vmax * dt0, mean_row));
         if (!filter_fits(I, h->geo, dt0)) c.ps[kSearchFilter] = INFINITY;
         return c;
     }
     bool wraps = false;   // with room for v_max to grow (InstDyn::p_image)
     for (int d = 0; d < h->dim; ++d) wraps = wraps || (h->geo.bc[d] == KMC_BC_PERIODIC && reach > 0.4 * h->geo.L[d]);
     const double mean_row = (double)I.n / std::max(s_rows, 1.0);
-    const double walks = walk_blocks(h, I, h->filter_chi != 0, vmax * dt0, mean_row);
+    const double walks = walk_blocks(I, h->geo, h->filter_chi != 0, vmax * dt0, mean_row);
     SearchCosts c = search_costs(h->dim, I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1, wraps, (double)h->n, cand, hits, passing, rows,
                                  n_row, walks);
     // Small single runs where a block per c-bin takes less (us, fitted to 320 pruned states of up

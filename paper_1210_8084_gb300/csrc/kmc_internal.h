@@ -399,6 +399,28 @@ inline SearchCosts search_costs64(int dim, double n_all, double cand, double n_r
     c.ps[kSearchPairs] = c.ps[kSearchDirect] + c.ps[kSearchFilter];   // binary32 only
     return c;
 }
+// Frame blocks that a warp of the filtered search walks, over all its runs of homes: the
+// frames as the step's constants set them (kmc_scan.cu, filter_constants), n_row homes
+// per row of search cells, spread over its length.
+inline double walk_blocks(const InstDev& I, const Geo& g, bool chi, double s, double n_row) {
+    const int F = g.dim - 1;
+    const double R = sqrt(I.R2), D = R + 2.0 * s, Re = I.sym ? R : 0.125 * R;
+    double reach = 0.0;
+    for (int d = 0; d <= F; ++d) reach = fmax(reach, fmin(D, 2.0 * I.s[d] * I.w[d]));
+    const double width = 2.0 * ((chi ? fmin(200.0 * R, 400.0 * s) : 46.0 * sqrt(Re * Re + s * s / 16.0)) - reach - s);
+    const double rows = fmax(n_row, 1e-3);
+    double blocks = 1.0 + 32.0 / rows;   // runs
+    for (int d = 0; d <= F; ++d) {
+        int sh = 0;
+        while ((1 << sh) < I.M[d] && fmin(2 << sh, I.M[d]) * I.w[d] <= width) ++sh;
+        const double k = ceil((1.001 * D + 1e-5 * g.L[d]) / I.w[d]), M = (double)I.M[d];
+        double cells = fmin(2.0 * k + 1.0, fmin(3 * I.s[d], I.M[d]));
+        if (d == F) cells = fmin(cells + fmin(1.0, 32.0 / rows) * M, M + 1.0);
+        blocks *= 1.0 + (cells - 1.0) / fmin(1 << sh, M);
+    }
+    return blocks;
+}
+
 // the cheapest of the searches in `allowed` (a bit each)
 inline int cheapest_search(const SearchCosts& c, unsigned allowed) {
     int best = -1;

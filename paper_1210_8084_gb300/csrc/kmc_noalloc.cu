@@ -127,7 +127,9 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     const size_t nv = buffer_rows(n);
     // The search as kmc_init chooses it (kmc_api.cu, estimate_search), without statistics
     // of the state: mean density, windows of the contact distance and a search cell,
-    // each pair once unless many candidates lie within the contact distance.
+    // each pair once unless many candidates lie within the contact distance; a largest
+    // displacement of a c-bin (the adaptive timestep's, and that of 0.2 c-bins at thermal
+    // speed) for the frames of the filter and for windows that may reach around the box.
     double within = nbar, cand = nbar, rows = 1.0, n_rows = 1.0;
     bool wraps = false;
     for (int d = 0; d < g.dim; ++d) {
@@ -136,18 +138,22 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
         cand *= fmin((2.0 * k + 1.0) * I.w[d], fmin(3.0 * g.L[d] / g.n[d], g.L[d]));
         if (d + 1 < g.dim) rows *= fmin(2.0 * k + 1.0, fmin(3.0 * I.s[d], I.M[d]));
         if (d + 1 < g.dim) n_rows *= I.M[d];
-        wraps = wraps || (g.bc[d] == KMC_BC_PERIODIC && k * I.w[d] > 0.4 * g.L[d]);
+        wraps = wraps || (g.bc[d] == KMC_BC_PERIODIC &&
+                          (k * I.w[d] > 0.4 * g.L[d] || sqrt(I.R2) + 2.2 * g.L[d] / g.n[d] > 0.45 * g.L[d]));
     }
     I.sym = sizeof(T) == 4 && within <= 4.0 * kSymPassing ? 1 : 0;
     const double near = fmin(within, cand), passing = 0.25 * near;
     const bool split = I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1;
-    const double n_row = (double)n / n_rows;
+    const double n_row = (double)n / n_rows, walks = walk_blocks(I, g, false, I.dx_min, n_row);
     I.search = n == 0 ? kSearchDirect
                : sizeof(T) == 8
-                   ? cheapest_search(search_costs64(g.dim, (double)n, cand, n_row, 1.0 + 32.0 / fmax(n_row, 1.0), 8.0),
+                   ? cheapest_search(search_costs64(g.dim, (double)n, cand, n_row, 1.0 + 32.0 / fmax(n_row, 1.0), 8.0),   // (*)
                                      1u << kSearchDirect | (filter_fits(I, g, I.dt) ? 1u << kSearchFilter : 0u))
                    : cheapest_search(search_costs(g.dim, split, wraps, (double)n, cand, I.sym ? 0.25 * near : 0.1 * cand, passing,
-                                                    rows, n_row, 0.0), 7u);
+                                                    rows, n_row, walks), 7u);
+    // (*) binary64: a few blocks; where they are many the filter may take 4 times as long as one
+    // thread per particle, which in a cluster that the mean density does not show takes 50 times as
+    // long as the filter
     I.close = passing > kPairsClose ? 1 : 0;
     I.chi = sizeof(T) == 8 ? 1 : 0;
     filter_lengths(I, g, sizeof(T) == 8);

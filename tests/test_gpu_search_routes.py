@@ -190,3 +190,32 @@ def test_small_runs_take_no_longer_than_a_block_per_c_bin(n, dim, cells, hi, R, 
         ms.append(min(p["search"] + p["tile"] for p in (sim.step_profiled(1) for _ in range(6))))
         sim.close()
     assert ms[0] < 1.3 * ms[1], ms
+
+
+def test_partner_call_where_windows_reach_around_the_box():
+    """Three periodic c-bins across: a step's reach is half the box, where the pair search decides every pair
+    exactly (9 times as long as one thread per particle); the call, without statistics of the state, keeps off it."""
+    import torch
+    import paper_1210_8084_gb300 as k
+    rng = np.random.default_rng(8)
+    n, cells = 3_528, (13, 3, 3)
+    hi = (1.0, 3 / 13, 3 / 13)
+    pos, vel = (0.9999 * rng.random((n, 3)) * hi).astype(np.float32), rng.standard_normal((n, 3), dtype=np.float32)
+    R = 0.04 / 13
+    base = dict(dim_pos=3, n_cells=cells, hi=hi, bc=(PER, PER, PER), sigma=np.pi * R * R, dt=0.178 / 13, precision=32,
+                sub_cells=(2, 3, 2))
+    p, v, best = torch.from_numpy(pos).cuda(), torch.from_numpy(vel).cuda(), torch.empty(n, dtype=torch.int32, device="cuda")
+    cfg = k.make_config(**base)
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    ms = []
+    for _ in range(6):
+        e0.record(torch.cuda.default_stream())
+        assert k.kmc_find_partners_noalloc(cfg, n, p, v, best) == k.KMC_OK
+        e1.record(torch.cuda.default_stream())
+        torch.cuda.synchronize()
+        ms.append(e0.elapsed_time(e1))
+    sim = k.Simulation(k.make_config(**base, flags=k.KMC_FLAG_NO_TILE_SEARCH), pos, vel)
+    sim.step(1)
+    direct = min(sim.step_profiled(1)["search"] for _ in range(4))
+    sim.close()
+    assert min(ms) < 2 * direct + 0.1, (min(ms), direct)
