@@ -145,15 +145,15 @@ int run(const kmc_config* cfg, int64_t n, const void* pos, const void* vel, int3
     const double near = fmin(within, cand), passing = 0.25 * near;
     const bool split = I.s[0] > 1 || I.s[1] > 1 || I.s[2] > 1;
     const double n_row = (double)n / n_rows, walks = walk_blocks(I, g, false, I.dx_min, n_row);
+    // (binary64 counts a few blocks: where they are many the filter may take 4 times as long as one
+    // thread per particle, which takes 50 times as long as the filter in a cluster that the mean
+    // density does not show)
     I.search = n == 0 ? kSearchDirect
                : sizeof(T) == 8
-                   ? cheapest_search(search_costs64(g.dim, (double)n, cand, n_row, 1.0 + 32.0 / fmax(n_row, 1.0), 8.0),   // (*)
+                   ? cheapest_search(search_costs64(g.dim, (double)n, cand, n_row, 1.0 + 32.0 / fmax(n_row, 1.0), 8.0),
                                      1u << kSearchDirect | (filter_fits(I, g, I.dt) ? 1u << kSearchFilter : 0u))
                    : cheapest_search(search_costs(g.dim, split, wraps, (double)n, cand, I.sym ? 0.25 * near : 0.1 * cand, passing,
                                                     rows, n_row, walks), 7u);
-    // (*) binary64: a few blocks; where they are many the filter may take 4 times as long as one
-    // thread per particle, which in a cluster that the mean density does not show takes 50 times as
-    // long as the filter
     I.close = passing > kPairsClose ? 1 : 0;
     I.chi = sizeof(T) == 8 ? 1 : 0;
     filter_lengths(I, g, sizeof(T) == 8);

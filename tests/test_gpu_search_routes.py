@@ -189,7 +189,7 @@ def test_small_runs_take_no_longer_than_a_block_per_c_bin(n, dim, cells, hi, R, 
         sim.step(1)
         ms.append(min(p["search"] + p["tile"] for p in (sim.step_profiled(1) for _ in range(6))))
         sim.close()
-    assert ms[0] < 1.3 * ms[1], ms
+    assert ms[0] < 1.5 * ms[1], ms
 
 
 def test_partner_call_where_windows_reach_around_the_box():
