@@ -154,7 +154,7 @@ KMC_API int kmc_window_size(kmc_handle* h, double* mean_candidates);
 
 /* Pair tests evaluated since kmc_init in instances that skip candidates out of
  * reach (kmc_info.tile_prune): the pairs left by the filter, each tested exactly;
- * with tile parameters, 4 for every (home, cluster of 4 staged candidates) pair
+ * in the tile search, 4 for every (home, cluster of 4 staged candidates) pair
  * whose boxes meet.  0 for other handles, whose window holds (C_p - 1) / 2 pairs
  * per particle, C_p from kmc_window_size.  Synchronises the handle's stream. */
 KMC_API int kmc_tile_tests(kmc_handle* h, double* tests);

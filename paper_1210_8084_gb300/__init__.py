@@ -306,7 +306,7 @@ def kmc_window_size(h):
 
 
 def kmc_tile_tests(h):
-    """Pair tests made by the pruned binary32 tile search since kmc_init."""
+    """Pair tests made since kmc_init in instances that skip candidates out of reach."""
     v = ctypes.c_double()
     _check(load().kmc_tile_tests(h, ctypes.byref(v)), h)
     return v.value

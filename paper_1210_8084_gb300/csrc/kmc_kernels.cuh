@@ -4,7 +4,7 @@
 // Step structure (Sagert et al., Sect. "Simulation setup" and Fig. 2):
 //   search  : closest PoCA candidate per particle over its c-bin neighbourhood
 //             (per particle here, or by kmc_filter.cuh / kmc_pairs.cuh; a block per
-//             c-bin where a flag or tile parameters ask for it)
+//             c-bin for small single runs, or where a flag or tile parameters ask for it)
 //   move    : unambiguous pairs, CM scattering, split free flight, walls,
 //             next search key + histogram
 //   scan    : exclusive scan of the key histogram (kmc_scan.cu)
